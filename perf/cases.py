@@ -39,16 +39,15 @@ def listed():
         # 20-cycle traces kept (plots, a hand-written optimiser's inner loop)
         dict(name="forward_c1_64", kind="forward", load="c1", modes=1, P=64, steps=4000,
              defl=True, f64=False),
-        # traces of a set of candidates of the 3-mode cantilever over a whole
-        # record, an odd number of them
-        dict(name="forward_c2_trace", kind="forward", load="c2", modes=3, P=1001, steps=25600,
+        # traces of a set of viscoelastic candidates (a law with a rate term)
+        # over a whole record, an odd number of them
+        dict(name="forward_c4_trace", kind="forward", load="c4", modes=3, P=1001, steps=25600,
              defl=True, f64=False),
         # a wide scan of the parameter cube, misfits only
         dict(name="forward_c2_wide", kind="forward", load="c2", modes=3, P=262144, steps=6400,
              defl=False, f64=False),
-        # the swarm of the paper's spring-damper experiment: 8 modes, a law
-        # with a rate term
-        dict(name="forward_f2_8modes", kind="forward", load="f2_spring_damper", modes=8, P=512,
+        # the swarm of the paper's own experiment: 8 modes, 8 cycles
+        dict(name="forward_f2_8modes", kind="forward", load="f2_hooke", modes=8, P=512,
              steps=4096, defl=False, f64=False),
         # reference traces in 64 bits (truths, checks of an inversion's result)
         dict(name="forward_c2_f64", kind="forward", load="c2", modes=3, P=96, steps=10240,
@@ -84,10 +83,13 @@ def draw(rng):
                        "fe", "misfit"])
     if kind in ("forward", "forward64"):
         f64 = kind == "forward64"
-        load = rng.choice(["c1", "c2", "c4", "f2_hooke", "f2_spring_damper"])
-        modes = 1 if load == "c1" else rng.choice([1, 2, 3, 3, 5, 8])
-        steps = _log_int(rng, 500, 10000 if f64 else 25600)
-        P = _log_int(rng, 16, 128) if f64 else _log_int(rng, 48, min(200000, 8e8 / steps))
+        load = rng.choice(["c1", "c2", "c2", "c4", "f2_hooke"])
+        f2 = load == "f2_hooke"
+        # the highest mode a step of 1/256 cycle resolves is the fifth or sixth
+        modes = 1 if load == "c1" else rng.choice([1, 3, 5, 8] if f2 else [1, 2, 3, 3, 5])
+        steps = _log_int(rng, 500, 4096 if f2 else 10000 if f64 else 25600)
+        P = _log_int(rng, 16, 128) if f64 else _log_int(
+            rng, 48, 4000 if f2 else min(200000, 8e8 / steps))
         defl = rng.random() < 0.5 and P * steps < 30e6
         return dict(kind="forward", load=load, modes=modes, P=P, steps=steps, defl=defl, f64=f64)
     if kind == "normal":
@@ -105,7 +107,7 @@ def draw(rng):
         load = rng.choice(["c1", "c2", "c4", "f2_hooke"])
         return dict(kind="invert", load=load, modes={"c1": 1, "f2_hooke": 8}.get(load, 3),
                     P=_log_int(rng, 64, 1500), iters=rng.randint(1, 5),
-                    steps=_log_int(rng, 1000, 20000))
+                    steps=_log_int(rng, 1000, 4096 if load == "f2_hooke" else 20000))
     if kind == "batch":
         lo = _log_int(rng, 600, 5000)
         return dict(kind="batch", load="c3", modes=rng.choice([1, 3, 3]),
