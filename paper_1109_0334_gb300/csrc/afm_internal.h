@@ -52,10 +52,57 @@ struct Coef {
     T c0, c1, c2, c3;
 };
 
+// The RK4 step of the modal cantilever as an affine map (host set-up:
+// affine_setup).  Between the four tip forces F1..F4 of a step everything is
+// linear, so the stage gaps and the step's increments are fixed combinations
+// of the state, the earlier stage forces and drive terms that depend only on
+// the phase: the classic stages (Eq. 2, Sec. 3.2) with the algebra done once
+// per problem in FP64 instead of once per step in the kernel.
+//
+// State per mode: the deflection q and a second coordinate,
+//   mode 0   w = B v + A1 q, the part of the step's increment of q that is
+//            linear in the state: q' - q = w + (forces, drive), and
+//            w' - w = c (q + w) + ec w + ...; ec = det - 1 alone carries the
+//            damping and c (with a low word) the frequency of the resonant
+//            mode, so that FP32 coefficients keep both to ~1e-8 relative
+//   others   p = 3 v (robust at any omega h; mode 0's form is singular where
+//            B = 0), with A1, B, C, D1 of the 2 x 2 step matrix rounded
+//            together so that its frequency and damping keep ~1e-9
+// Stage gaps: d1 = zq + s1, d2 = zq + (s1 + ...), with zq = Zc + q_0 and
+// the small remainders summed first; d3, d4 add e31 F1 and e41 F1 + e42 F2.
+#define AFM_AFF_TAB 24   // drive terms per phase, at most (8 modes, rate law: 21)
+template <typename T>
+struct Affine {
+    T d2q, d2w;                              // stage 2 of mode 0 beyond q_0
+    T d3q[AFM_MAXM], d3p[AFM_MAXM];          // stage 3, 4 gaps (mode 0: beyond q_0)
+    T d4q[AFM_MAXM], d4p[AFM_MAXM];
+    T e31, e41, e42;
+    T ec, c0, c0lo;                          // mode 0's second coordinate
+    T A1[AFM_MAXM], B[AFM_MAXM], C[AFM_MAXM], D1[AFM_MAXM];   // modes >= 1
+    T bq[3][AFM_MAXM], bp[4][AFM_MAXM];      // increments per unit stage force
+    // gap rates of the stages (laws with a rate term); stage 1:
+    // v1q q_0 + v1w w_0 + (sum of p_i) / 3
+    T v1q, v1w, third;
+    T r2q[AFM_MAXM], r2p[AFM_MAXM], r3q[AFM_MAXM], r3p[AFM_MAXM], r4q[AFM_MAXM], r4p[AFM_MAXM];
+    T h21, h31, h32, h41, h42, h43;
+    T p0[AFM_MAXM];                          // initial second coordinates
+    // drive term k at phase j: dS[k] sin(2 pi j / spc) + dC[k] cos(2 pi j / spc);
+    // k = 0, 1: gaps of stages 3, 4; 2 + i, 2 + M + i: increments of q_i and
+    // of the second coordinate (M: the kernels' template mode count);
+    // 2 + 2 M ..: gap rates of stages 2, 3, 4
+    double dS[AFM_AFF_TAB], dC[AFM_AFF_TAB];
+};
+
+// Template mode count of the kernels for m modes (modes past m have zero
+// constants), and the words per phase of their drive-term rows.
+AFM_HD constexpr int aff_modes(int m) { return (m == 1 || m == 3) ? m : AFM_MAXM; }
+AFM_HD constexpr int aff_row(int M, bool rate) { return (2 + 2 * M + (rate ? 3 : 0) + 3) & ~3; }
+
 // Constants of one problem in the arithmetic type of a kernel (float or
 // double), filled on the host by the per-problem set-up.
 template <typename T>
 struct KConst {
+    Affine<T> af;
     T w2[AFM_MAXM], w2lo[AFM_MAXM], wq[AFM_MAXM], gam[AFM_MAXM], tip[AFM_MAXM];
     T cmask[AFM_MAXM];              // 1: mode i takes compensated sums (comp_mode), else 0
     T q0[AFM_MAXM], v0[AFM_MAXM];

@@ -171,6 +171,184 @@ void modal_setup(const afm_problem& pr, int spc, Setup& s) {
     s.h = 1.0 / (pr.f1_hz * spc);
 }
 
+// ---------------------------------------------------------------------------
+// The RK4 step as an affine map (Affine in afm_internal.h): every stage value
+// of one mode as a linear form of [q, v, F1, F2, F3, F4, g0, gh, g1].
+// ---------------------------------------------------------------------------
+struct Lin {
+    double c[9];
+};
+Lin lin_unit(int k) {
+    Lin l{};
+    l.c[k] = 1.0;
+    return l;
+}
+Lin operator+(const Lin& a, const Lin& b) {
+    Lin r;
+    for (int i = 0; i < 9; ++i) r.c[i] = a.c[i] + b.c[i];
+    return r;
+}
+Lin operator*(double s, const Lin& a) {
+    Lin r;
+    for (int i = 0; i < 9; ++i) r.c[i] = s * a.c[i];
+    return r;
+}
+
+// FP32 values of a mode's step matrix I + [A1 B; C D1], chosen among the
+// floats within two ulps of each entry so that the errors of its frequency
+// and damping cancel.  Rounded one by one they are off by ~3e-8 theta^2 per
+// step, which shifts the damping theta / Q of a fast mode by a few 1e-6: the
+// deflections of the paper's 8-mode experiment then end 1.4 times further
+// from FP64 than those of the classic stages, and 0.6 times as far with this
+// choice.
+void round_step_matrix(const double ex[4], float out[4]) {
+    constexpr int R = 2, N = 2 * R + 1;
+    float cand[4][N];
+    for (int k = 0; k < 4; ++k) {
+        out[k] = cand[k][R] = (float)ex[k];
+        for (int r = 1; r <= R; ++r) {
+            cand[k][R + r] = std::nextafterf(cand[k][R + r - 1], 1e30f);
+            cand[k][R - r] = std::nextafterf(cand[k][R - r + 1], -1e30f);
+        }
+    }
+    const double A = 1.0 + ex[0], B = ex[1], C = ex[2], D = 1.0 + ex[3];
+    const double det = A * D - B * C, tr = A + D;
+    if (!(det > 0.0)) return;
+    const double ct = tr / (2.0 * std::sqrt(det));
+    if (!(std::fabs(ct) < 0.9999999)) return;
+    // errors of ln(damping) and of the angle, to first order
+    const double gd = 0.5 / det, ist = 1.0 / std::sqrt(1.0 - ct * ct);
+    const double tt = ist / (2.0 * std::sqrt(det)), td = ist * tr / (4.0 * det * std::sqrt(det));
+    double best = 1e300;
+    for (int a = 0; a < N; ++a)
+        for (int d = 0; d < N; ++d) {
+            const double ea = cand[0][a] - ex[0], ed = cand[3][d] - ex[3];
+            const double t = ea + ed, d0 = D * ea + A * ed;
+            for (int b = 0; b < N; ++b) {
+                const double eb = cand[1][b] - ex[1], d1 = d0 - C * eb;
+                for (int c = 0; c < N; ++c) {
+                    const double ec = cand[2][c] - ex[2];
+                    const double dd = d1 - B * ec - eb * ec;
+                    const double g = gd * dd, th = tt * t - td * dd;
+                    const double err = g * g + th * th;
+                    if (err < best) {
+                        best = err;
+                        out[0] = cand[0][a];
+                        out[1] = cand[1][b];
+                        out[2] = cand[2][c];
+                        out[3] = cand[3][d];
+                    }
+                }
+            }
+        }
+}
+
+// w2, wq, gam: the modes' scaled constants in FP64; q0, v0: initial state;
+// amp, phase: the drive g = amp sin(2 pi j / (2 spc) + phase) at half step j.
+template <typename T>
+void affine_setup(int m, const double* w2, const double* wq, const double* gam, const double* q0,
+                  const double* v0, double amp, double phase, int spc, afm::Affine<T>& A) {
+    std::memset(&A, 0, sizeof(A));
+    const int M = afm::aff_modes(m);
+    double e31 = 0, e41 = 0, e42 = 0, h[6] = {0, 0, 0, 0, 0, 0};
+    double tab[AFM_AFF_TAB][3] = {};
+    for (int i = 0; i < m; ++i) {
+        auto acc = [&](const Lin& q, const Lin& v, int f, int g) {
+            return (-w2[i]) * q + (-wq[i]) * v + lin_unit(f) + gam[i] * lin_unit(g);
+        };
+        const Lin q = lin_unit(0), v = lin_unit(1);
+        const Lin a1 = acc(q, v, 2, 6);
+        const Lin v2 = v + 3.0 * a1, a2 = acc(q + 3.0 * v, v2, 3, 7);
+        const Lin v3 = v + 3.0 * a2, a3 = acc(q + 3.0 * v2, v3, 4, 7);
+        const Lin v4 = v + 6.0 * a3, a4 = acc(q + 6.0 * v3, v4, 5, 8);
+        const Lin dq = v + 2.0 * v2 + 2.0 * v3 + v4, dv = a1 + 2.0 * a2 + 2.0 * a3 + a4;
+        // second coordinate = pq q + pv v
+        const double pq = i == 0 ? dq.c[0] : 0.0, pv = i == 0 ? dq.c[1] : 3.0;
+        auto coord = [&](const Lin& l) {   // a form in (q, v) as one in (q, second coordinate)
+            Lin r = l;
+            r.c[1] = l.c[1] / pv;
+            r.c[0] = l.c[0] - l.c[1] * (pq / pv);
+            return r;
+        };
+        const Lin self = i == 0 ? 0.0 * q : q;   // mode 0: the stage gaps beyond q_0
+        const Lin g2 = coord(self + 3.0 * v), g3 = coord(self + 3.0 * v2),
+                  g4 = coord(self + 6.0 * v3);
+        const Lin Dq = coord(dq), Dp = coord(pq * dq + pv * dv);
+        const Lin r2 = coord(v2), r3 = coord(v3), r4 = coord(v4);
+        if (i == 0) {
+            A.d2q = (T)g2.c[0];
+            A.d2w = (T)g2.c[1];
+            A.ec = (T)(Dp.c[1] - Dp.c[0]);
+            A.c0 = (T)Dp.c[0];
+            A.c0lo = (T)(Dp.c[0] - (double)A.c0);
+            A.v1q = (T)(-pq / pv);
+            A.v1w = (T)(1.0 / pv);
+        } else {
+            const double ex[4] = {Dq.c[0], Dq.c[1], Dp.c[0], Dp.c[1]};
+            if (sizeof(T) == 4) {
+                float f[4];
+                round_step_matrix(ex, f);
+                A.A1[i] = (T)f[0];
+                A.B[i] = (T)f[1];
+                A.C[i] = (T)f[2];
+                A.D1[i] = (T)f[3];
+            } else {
+                A.A1[i] = (T)ex[0];
+                A.B[i] = (T)ex[1];
+                A.C[i] = (T)ex[2];
+                A.D1[i] = (T)ex[3];
+            }
+        }
+        A.d3q[i] = (T)g3.c[0];
+        A.d3p[i] = (T)g3.c[1];
+        A.d4q[i] = (T)g4.c[0];
+        A.d4p[i] = (T)g4.c[1];
+        e31 += g3.c[2];
+        e41 += g4.c[2];
+        e42 += g4.c[3];
+        for (int k = 0; k < 3; ++k) A.bq[k][i] = (T)Dq.c[2 + k];
+        for (int k = 0; k < 4; ++k) A.bp[k][i] = (T)Dp.c[2 + k];
+        A.r2q[i] = (T)r2.c[0];
+        A.r2p[i] = (T)r2.c[1];
+        A.r3q[i] = (T)r3.c[0];
+        A.r3p[i] = (T)r3.c[1];
+        A.r4q[i] = (T)r4.c[0];
+        A.r4p[i] = (T)r4.c[1];
+        h[0] += r2.c[2];
+        h[1] += r3.c[2];
+        h[2] += r3.c[3];
+        h[3] += r4.c[2];
+        h[4] += r4.c[3];
+        h[5] += r4.c[4];
+        A.p0[i] = (T)(pq * q0[i] + pv * v0[i]);
+        for (int k = 0; k < 3; ++k) {
+            tab[0][k] += g3.c[6 + k];
+            tab[1][k] += g4.c[6 + k];
+            tab[2 + i][k] = Dq.c[6 + k];
+            tab[2 + M + i][k] = Dp.c[6 + k];
+            tab[2 + 2 * M][k] += r2.c[6 + k];
+            tab[3 + 2 * M][k] += r3.c[6 + k];
+            tab[4 + 2 * M][k] += r4.c[6 + k];
+        }
+    }
+    A.third = (T)(1.0 / 3.0);
+    A.e31 = (T)e31;
+    A.e41 = (T)e41;
+    A.e42 = (T)e42;
+    A.h21 = (T)h[0];
+    A.h31 = (T)h[1];
+    A.h32 = (T)h[2];
+    A.h41 = (T)h[3];
+    A.h42 = (T)h[4];
+    A.h43 = (T)h[5];
+    for (int k = 0; k < AFM_AFF_TAB; ++k)
+        for (int t = 0; t < 3; ++t) {
+            const double ph = phase + t * kPi / spc;
+            A.dS[k] += tab[k][t] * amp * std::cos(ph);
+            A.dC[k] += tab[k][t] * amp * std::sin(ph);
+        }
+}
+
 template <typename T>
 void fill_kconst(const afm_problem& pr, int spc, int n_steps, KConst<T>& K) {
     Setup s;
@@ -195,6 +373,16 @@ void fill_kconst(const afm_problem& pr, int spc, int n_steps, KConst<T>& K) {
     K.Zc = (T)(pr.Zc_m / nm);
     K.drive_amp = (s.a / nm) * (s.wd * tau) * (s.wd * tau);
     K.drive_phase = s.psi;
+    if (!drv) {
+        double w2[AFM_MAXM], wq[AFM_MAXM], q0[AFM_MAXM], v0[AFM_MAXM];
+        for (int i = 0; i < s.m; ++i) {
+            w2[i] = (s.w[i] * tau) * (s.w[i] * tau);
+            wq[i] = s.w[i] * tau / pr.Q[i];
+            q0[i] = s.q0[i] / nm;
+            v0[i] = s.v0[i] * tau / nm;
+        }
+        affine_setup(s.m, w2, wq, s.gam, q0, v0, K.drive_amp, K.drive_phase, spc, K.af);
+    }
     K.m = s.m;
     K.spc2 = 2 * spc;
     K.n_steps = n_steps;

@@ -144,10 +144,6 @@ cudaError_t launch_forward_f32(const KConst<float>& K, const float* x, int P, fl
         return launch_forward_x2(K, x, P, defl, U, S, flags, st);
     return launch_forward<float>(K, x, P, defl, U, S, flags, st);
 }
-cudaError_t launch_forward_f64(const KConst<double>& K, const double* x, int P, double* defl,
-                               const double* U, double* S, int* flags, cudaStream_t st) {
-    return launch_forward<double>(K, x, P, defl, U, S, flags, st);
-}
 
 // ---------------------------------------------------------------------------
 // Standalone misfit (Eq. 5) of a time-major deflection array.  HBM-bound:
