@@ -97,6 +97,9 @@ struct Affine {
 // constants), and the words per phase of their drive-term rows.
 AFM_HD constexpr int aff_modes(int m) { return (m == 1 || m == 3) ? m : AFM_MAXM; }
 AFM_HD constexpr int aff_row(int M, bool rate) { return (2 + 2 * M + (rate ? 3 : 0) + 3) & ~3; }
+// words per phase of an FP64 table (aff::Table<double>)
+AFM_HD constexpr int aff_row64(int M, bool rate) { return M > 3 ? 2 : aff_row(M, rate); }
+AFM_HD constexpr bool rate_law(int force) { return force == 2 || force == 4; }
 
 // Constants of one problem in the arithmetic type of a kernel (float or
 // double), filled on the host by the per-problem set-up.

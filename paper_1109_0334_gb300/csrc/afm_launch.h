@@ -46,18 +46,20 @@ cudaError_t launch_synth(const KConst<float>& K, const double* x_truth, int n_pi
 
 // Per-pixel problem constants of a batch whose pixels differ in their
 // cantilever or set-point (afm_problem per pixel): indexed by pixel id, with
-// each pixel's drive table at its 2 spc half-step phases (+ wrap entry) in
-// FP64 and rounded to FP32.  kf == nullptr: every pixel uses the launch's
-// constants.
+// each pixel's drive g at its 2 spc half-step phases (+ wrap entry) in FP32
+// and the drive terms of the affine step: FP32 rows and the FP64 sine and
+// cosine of each phase (tab64).  kf == nullptr: every pixel uses the launch's constants.
 struct PixConst {
     const KConst<float>* kf;    // [n_pix]
     const KConst<double>* kd;   // [n_pix]
-    const double* tab64;        // [n_pix][ld]
+    const double* tab64;        // [n_pix][ld64]
     const float* tab32;         // [n_pix][ld]
-    int ld;
+    const float* rows;          // [n_pix][ld_rows]
+    int ld, ld64, ld_rows;
 };
-// fills tab64 / tab32 of n_pix pixels from kd (the formula of build_drive_table)
-cudaError_t launch_pix_tables(const PixConst& pc, int n_pix, int spc2, cudaStream_t st);
+// fills the tables of n_pix pixels from kd and kf
+cudaError_t launch_pix_tables(const PixConst& pc, int m, int force, int n_pix, int spc2,
+                              cudaStream_t st);
 
 // many independent pixel inversions in one persistent launch
 struct BatchArgs {
@@ -241,7 +243,7 @@ struct ReevalWinner {
 };
 struct ReevalPtrs {
     ReevalWinner* win;
-    double* tab;          // [spc2 + 1] FP64 drive table
+    double* tab;          // [2 spc] sine and cosine of the phases (room for spc2 + 1)
     double* start[2];     // [B + 1][2m] segment start states (alternating sweeps)
     double* E;            // [B][2m] segment end states
     double* J;            // [B][2m][2m] segment tangent maps
@@ -253,7 +255,7 @@ struct ReevalPtrs {
 // owns segments [i maxB, (i + 1) maxB) of the segment arrays.
 struct ReevalBatch {
     double* coef;   // [n_pix][4] FP64 force coefficients of each slot's winner
-    double* tab;    // [spc2 + 1] FP64 drive table
+    double* tab;    // FP64 drive terms of every phase (aff::Table)
     double* Z;      // [n_pix * maxB][2m] segment start states (corrected in place)
     double* E;      // [n_pix * maxB][2m] segment end states
     float* J;       // [n_pix * maxB][2m][2m] segment tangent maps (FP32)
@@ -261,8 +263,9 @@ struct ReevalBatch {
     double* u2;     // [n_pix] sum of U^2 of each slot's record
     int maxB;       // segments of the longest record (problem n_steps)
 };
-size_t reeval_batch_bytes(int m, int n_steps, int spc, int n_pix);
-void reeval_batch_carve(void* base, int m, int n_steps, int spc, int n_pix, ReevalBatch* R);
+size_t reeval_batch_bytes(int m, int force, int n_steps, int spc, int n_pix);
+void reeval_batch_carve(void* base, int m, int force, int n_steps, int spc, int n_pix,
+                        ReevalBatch* R);
 // fills each slot's result record (S_f64, J_rel, theta, status, defect,
 // segments) from the parameters already in it
 cudaError_t launch_reeval_batch(const KConst<float>& Kf, const KConst<double>& Kd,

@@ -6,6 +6,7 @@
 
 #include <type_traits>
 
+#include "afm_affine.cuh"
 #include "afm_device.cuh"
 #include "afm_launch.h"
 
@@ -41,80 +42,95 @@ cudaError_t dispatch_m13(int m, int force, F&& f) {
     return cudaErrorInvalidValue;
 }
 
-// Modal accelerations of one FP64 stage (the arithmetic of accel<double>),
-// also returning the gap d and its rate d'.
-template <int M, int FORCE>
-__device__ __forceinline__ void accel64(const KConst<double>& K, const Coef<double>& c,
-                                        const double* q, const double* v, double g, double* a,
-                                        double& d, double& dd) {
-    double u = q[0];
-#pragma unroll
-    for (int i = 1; i < M; ++i) u += q[i];
-    dd = 0.0;
-    if (UsesRate<FORCE>::value) {
-        dd = v[0];
-#pragma unroll
-        for (int i = 1; i < M; ++i) dd += v[i];
-    }
-    d = K.Zc + u;
-    const double F = tip_force<FORCE, double>(c, d, dd);
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        double ai = fma(-K.wq[i], v[i], K.gam[i] * g);
-        ai = fma(-K.w2[i], q[i], ai);
-        a[i] = (M <= 4) ? ai + F : fma(K.tip[i], F, ai);   // tip 0: padding modes
-    }
-}
-
-// One FP64 RK4 step (the stage pattern of rk4_step, uncompensated: FP64
-// needs no compensation over a segment).  REC: the force slopes of each stage
-// go to rec[k * 32], k = 2 * stage (+1 for the rate slope).
+// One FP64 RK4 step in the affine form (afm_affine.cuh), uncompensated: FP64
+// needs no compensation over a segment.  R: the step's drive terms.  REC: the
+// force slopes of each stage go to rec[k * 32], k = 2 * stage (+1 for the rate
+// slope).
 template <int M, int FORCE, bool REC>
-__device__ __forceinline__ void step64(const KConst<double>& K, const Coef<double>& c,
-                                       const Coef<float>& cf, double* q, double* v, double g0,
-                                       double gh, double g1, float* rec) {
-    double a[M], qs[M], vs[M], Kq[M], Kv[M], d, dd;
-    auto slope = [&](int st) {
-        if (REC) {
+__device__ __forceinline__ void step64(const KConst<double>& K, const aff::LawCoef<double>& c,
+                                       const Coef<float>& cf, const double* R,
+                                       aff::State<double, M, aff::NONE>& s, float* rec) {
+    aff::Stages<double> g;
+    aff::stages<double, M, FORCE, aff::NONE>(K, c, R, s, g);
+    if constexpr (REC) {
+#pragma unroll
+        for (int st = 0; st < 4; ++st) {
             float Fd, Fr, Fc[4];
-            force_partials<FORCE>(cf, (float)d, (float)dd, Fd, Fr, Fc);
+            force_partials<FORCE>(cf, (float)g.d[st], (float)g.r[st], Fd, Fr, Fc);
             rec[(2 * st) * 32] = Fd;
             rec[(2 * st + 1) * 32] = Fr;
         }
-    };
-    accel64<M, FORCE>(K, c, q, v, g0, a, d, dd);
-    slope(0);
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        Kq[i] = v[i];
-        Kv[i] = a[i];
-        qs[i] = fma(3.0, v[i], q[i]);
-        vs[i] = fma(3.0, a[i], v[i]);
     }
-    accel64<M, FORCE>(K, c, qs, vs, gh, a, d, dd);
-    slope(1);
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        Kq[i] = fma(2.0, vs[i], Kq[i]);
-        Kv[i] = fma(2.0, a[i], Kv[i]);
-        qs[i] = fma(3.0, vs[i], q[i]);
-        vs[i] = fma(3.0, a[i], v[i]);
+    aff::advance<double, M, aff::NONE>(K, R, g.F, s);
+}
+
+// Drive terms of phase j.  COMPACT: tab holds the sine and cosine of each
+// phase (2 spc doubles), else the rows of build_rows.
+template <int M, int FORCE, bool COMPACT>
+__device__ __forceinline__ void drive_terms(const KConst<double>& K, const double* tab, int j,
+                                            double (&R)[aff::Rows<M, FORCE>::words]) {
+    if constexpr (COMPACT)
+        aff::phase_terms<M, FORCE>(K, tab[2 * j], tab[2 * j + 1], R);
+    else
+        aff::load_row<double, M, FORCE>(K, tab + (size_t)j * aff::Rows<M, FORCE>::words, R);
+}
+
+// The whole record by one thread: the fallback of both re-evaluations.
+template <int M, int FORCE, bool COMPACT>
+__device__ __forceinline__ double integrate64(const KConst<double>& K,
+                                              const aff::LawCoef<double>& c, const double* tab,
+                                              const float* __restrict__ U, int n) {
+    aff::State<double, M, aff::ALL> s;
+    aff::init<double, M, aff::ALL>(K, s);
+    double S = 0.0, cS = 0.0;
+    const int spc = K.spc2 >> 1;
+    int j = 0;
+    for (int t = 0; t < n; ++t) {
+        double R[aff::Rows<M, FORCE>::words];
+        drive_terms<M, FORCE, COMPACT>(K, tab, j, R);
+        if (++j == spc) j = 0;
+        aff::step<double, M, FORCE, aff::ALL>(K, c, R, s);
+        if (K.np > 0) {
+            for (int k = 0; k < K.np; ++k)
+                aff::misfit_add((double)U[(size_t)t * K.np + k], aff::point_defl(K, k, s), S, cS);
+        } else {
+            aff::misfit_add((double)U[t], aff::tip(s), S, cS);
+        }
     }
-    accel64<M, FORCE>(K, c, qs, vs, gh, a, d, dd);
-    slope(2);
+    return S;
+}
+
+// FP32 steps 0 .. n - 1 of the winner from rows in shared memory (every word
+// once); the FP64 value of the state after every AFM_SEG-th step goes to
+// Y[b][2m], b = 1 .. B - 1.  One warp's instruction stream bounds it (~130
+// per step): a step's drive terms are loaded during the step before.
+template <int M, int FORCE>
+__device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const KConst<double>& Kd,
+                                             const Coef<float>& cf, const float* rows, int n,
+                                             int B, double* Y) {
+    constexpr int S2 = 2 * M, W = aff::Rows<M, FORCE>::words;
+    const aff::LawCoef<float> c = aff::law_coef(cf);
+    aff::State<float, M, aff::MODE0> s;
+    aff::init<float, M, aff::MODE0>(Kf, s);
+    const float* row = rows;
+    const float* end = rows + (size_t)(Kf.spc2 >> 1) * W;
+    float R[W];
+    aff::load_row<float, M, FORCE>(Kf, row, R);
+    int b = 1, next = AFM_SEG;
+    for (int t = 0; t < n && b < B; ++t) {
+        row += W;
+        if (row == end) row = rows;
+        float Rn[W];
+        aff::load_row<float, M, FORCE>(Kf, row, Rn);
+        aff::step<float, M, FORCE, aff::MODE0>(Kf, c, R, s);
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-        Kq[i] = fma(2.0, vs[i], Kq[i]);
-        Kv[i] = fma(2.0, a[i], Kv[i]);
-        qs[i] = fma(6.0, vs[i], q[i]);
-        vs[i] = fma(6.0, a[i], v[i]);
-    }
-    accel64<M, FORCE>(K, c, qs, vs, g1, a, d, dd);
-    slope(3);
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        q[i] = q[i] + (Kq[i] + vs[i]);
-        v[i] = v[i] + (Kv[i] + a[i]);
+        for (int k = 0; k < W; ++k) R[k] = Rn[k];
+        if (t + 1 == next) {
+            aff::export_state<float, M, aff::MODE0>(Kd, s, Y + (size_t)b * S2,
+                                                    Y + (size_t)b * S2 + M);
+            ++b;
+            next += AFM_SEG;
+        }
     }
 }
 
@@ -140,7 +156,7 @@ __device__ __forceinline__ void jvp_stage(const float* w2, const float* wq, cons
     }
 }
 
-// The RK4 step of step64 linearised about its recorded stages, applied to one
+// The RK4 step (stage form, in q and v) linearised about its recorded stages, applied to one
 // tangent direction (dq, dv) in place.
 template <int M, int FORCE>
 __device__ __forceinline__ void jvp_step(const float* w2, const float* wq, const float* tip,

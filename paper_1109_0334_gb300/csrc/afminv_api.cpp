@@ -912,27 +912,31 @@ BatchLayout batch_layout(int n_pix) {
 // for the longest record, problem n_steps).
 size_t batch_ws_bytes(const afm_problem& pr, int n_run) {
     return batch_layout(n_run).total +
-           align256(afm::reeval_batch_bytes(problem_modes(pr), pr.n_steps, pr.steps_per_cycle,
+           align256(afm::reeval_batch_bytes(problem_modes(pr), pr.force, pr.n_steps, pr.steps_per_cycle,
                                             n_run));
 }
 
 // Per-pixel problems of a batch (an afm_problem per pixel): their constants
 // and drive tables at the end of the workspace, indexed by pixel id.
 struct PixLayout {
-    size_t kf, kd, t64, t32, total;
-    int ld;
+    size_t kf, kd, t64, t32, rows, total;
+    int ld, ld64, ld_rows;
 };
 
-PixLayout pix_layout(int n_prob, int spc) {
+PixLayout pix_layout(int n_prob, const afm_problem& pr) {
     PixLayout L{};
     if (n_prob <= 1) return L;
     const size_t n = (size_t)n_prob;
+    const int M = afm::aff_modes(problem_modes(pr)), spc = pr.steps_per_cycle;
     L.ld = (2 * spc + 1 + 3) & ~3;
+    L.ld64 = 2 * spc;
+    L.ld_rows = spc * afm::aff_row(M, afm::rate_law(pr.force));
     L.kf = 0;
     L.kd = align256(sizeof(KConst<float>) * n);
     L.t64 = L.kd + align256(sizeof(KConst<double>) * n);
-    L.t32 = L.t64 + align256(sizeof(double) * n * L.ld);
-    L.total = L.t32 + align256(sizeof(float) * n * L.ld);
+    L.t32 = L.t64 + align256(sizeof(double) * n * L.ld64);
+    L.rows = L.t32 + align256(sizeof(float) * n * L.ld);
+    L.total = L.rows + align256(sizeof(float) * n * L.ld_rows);
     return L;
 }
 
@@ -1760,7 +1764,7 @@ afm_status afm_invert_batch_workspace_size(const afm_problem* probs, int n_prob,
     afm_problem eff;
     afm_status st = check_batch_probs(probs, n_prob, n_pix, &eff);
     if (st) return st;
-    *bytes = batch_ws_bytes(eff, n_pix) + pix_layout(n_prob, eff.steps_per_cycle).total;
+    *bytes = batch_ws_bytes(eff, n_pix) + pix_layout(n_prob, eff).total;
     return AFM_OK;
 }
 
@@ -1807,7 +1811,7 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
     BatchSetup& B = *out;
     fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, B.Kf);
     fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, B.Kd);
-    afm::reeval_batch_carve(ws + L.total, problem_modes(*prob), prob->n_steps,
+    afm::reeval_batch_carve(ws + L.total, problem_modes(*prob), prob->force, prob->n_steps,
                             prob->steps_per_cycle, n_run, &B.R);
     B.pc = pso_const(*cfg, prob->n_free);
     afm::BatchArgs& a = B.a;
@@ -1837,7 +1841,7 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
     if (n_prob > 1) {
         // every pixel's constants (FP32 and FP64), uploaded to the workspace,
         // and its drive tables computed there
-        const PixLayout X = pix_layout(n_prob, prob->steps_per_cycle);
+        const PixLayout X = pix_layout(n_prob, *prob);
         char* pw = ws + pix_at;
         std::vector<KConst<float>> kf(n_prob);
         std::vector<KConst<double>> kd(n_prob);
@@ -1855,8 +1859,12 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
         a.pix.kd = reinterpret_cast<const KConst<double>*>(pw + X.kd);
         a.pix.tab64 = reinterpret_cast<const double*>(pw + X.t64);
         a.pix.tab32 = reinterpret_cast<const float*>(pw + X.t32);
+        a.pix.rows = reinterpret_cast<const float*>(pw + X.rows);
         a.pix.ld = X.ld;
-        AFM_CUDA(afm::launch_pix_tables(a.pix, n_prob, 2 * prob->steps_per_cycle, s),
+        a.pix.ld64 = X.ld64;
+        a.pix.ld_rows = X.ld_rows;
+        AFM_CUDA(afm::launch_pix_tables(a.pix, B.Kf.m, B.Kf.force, n_prob,
+                                        2 * prob->steps_per_cycle, s),
                  "per-pixel drive tables");
     }
     // queue order (longest record first) is needed by the tuner's probe too
@@ -1899,7 +1907,7 @@ afm_status afm_invert_batch(afm_ctx* ctx, const afm_problem* probs, int n_prob,
     afm_status st0;
     if ((st0 = check_batch_probs(probs, n_prob, n_pix, &eff))) return st0;
     const size_t pix_at = batch_ws_bytes(eff, n_pix);
-    const size_t need = pix_at + pix_layout(n_prob, eff.steps_per_cycle).total;
+    const size_t need = pix_at + pix_layout(n_prob, eff).total;
     if (workspace_bytes < need)
         return fail(AFM_ERR_INVALID_ARG, "workspace %zu bytes < %zu needed", workspace_bytes, need);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -2049,7 +2057,7 @@ afm_status afm_invert_batch_polished_workspace_size(const afm_problem* probs, in
     afm_problem eff;
     if ((st = check_batch_probs(probs, n_prob, n_prob > 1 ? n_prob : 1, &eff))) return st;
     *bytes = batch_polish_layout(eff, *cfg, n_run, polish_k, n_cand, method).total +
-             pix_layout(n_prob, eff.steps_per_cycle).total;
+             pix_layout(n_prob, eff).total;
     return AFM_OK;
 }
 
@@ -2078,7 +2086,7 @@ afm_status afm_invert_batch_polished(afm_ctx* ctx, const afm_problem* probs, int
         return fail(AFM_ERR_UNSUPPORTED,
                     "per-pixel problems are polished by Levenberg-Marquardt (AFM_POLISH_LM) only");
     const BatchPolishLayout PL = batch_polish_layout(eff, *cfg, n_run, polish_k, n_cand, method);
-    const size_t need = PL.total + pix_layout(n_prob, eff.steps_per_cycle).total;
+    const size_t need = PL.total + pix_layout(n_prob, eff).total;
     if (workspace_bytes < need)
         return fail(AFM_ERR_INVALID_ARG, "workspace %zu bytes < %zu needed", workspace_bytes, need);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);

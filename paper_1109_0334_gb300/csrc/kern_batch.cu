@@ -27,27 +27,47 @@ size_t batch_smem(int P, int D, int spc2, bool pp) {
 
 // ---------------------------------------------------------------------------
 // Per-pixel drive tables (batches whose pixels differ in their problem): the
-// arithmetic of build_drive_table in FP64 from each pixel's constants, also
-// rounded to FP32.  One thread per (pixel, phase).
+// FP32 half-step table (the arithmetic of build_drive_table) and the drive
+// terms of the affine step (that of build_rows).  One thread per (pixel,
+// phase).
 // ---------------------------------------------------------------------------
-__global__ void pix_tables_kernel(const KConst<double>* __restrict__ kd, int n_pix, int spc2,
-                                  int ld, double* __restrict__ tab64, float* __restrict__ tab32) {
+__global__ void pix_tables_kernel(const PixConst pc, int n_pix, int spc2, int words, int terms,
+                                  double* __restrict__ tab64,
+                                  float* __restrict__ tab32, float* __restrict__ rows) {
+    const int spc = spc2 >> 1;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int pix = (int)(t / (spc2 + 1)), j = (int)(t % (spc2 + 1));
+    const int pix = (int)(t / spc), j = (int)(t % spc);
     if (pix >= n_pix) return;
-    const int jj = j == spc2 ? 0 : j;
-    const double ph = 6.283185307179586476925 * (double)jj / (double)spc2 + kd[pix].drive_phase;
-    const double g = kd[pix].drive_amp * sin(ph);
-    tab64[(size_t)pix * ld + j] = g;
-    tab32[(size_t)pix * ld + j] = (float)g;
+    const KConst<float>& kf = pc.kf[pix];
+    const KConst<double>& kd = pc.kd[pix];
+    float* t32 = tab32 + (size_t)pix * pc.ld;
+    for (int h = 2 * j; h < 2 * j + 2; ++h) {
+        const double ph = 6.283185307179586476925 * (double)h / (double)spc2 + kd.drive_phase;
+        t32[h] = (float)(kd.drive_amp * sin(ph));
+    }
+    if (j == 0) t32[spc2] = t32[0];
+    double s, c;
+    sincospi((2.0 / (double)spc) * (double)j, &s, &c);
+    float* r32 = rows + (size_t)pix * pc.ld_rows + (size_t)j * words;
+    for (int k = 0; k < words; ++k)
+        r32[k] = k < terms ? (float)fma(kf.af.dS[k], s, kf.af.dC[k] * c) : 0.f;
+    double* r64 = tab64 + (size_t)pix * pc.ld64 + 2 * j;
+    r64[0] = s;
+    r64[1] = c;
 }
 
-cudaError_t launch_pix_tables(const PixConst& pc, int n_pix, int spc2, cudaStream_t st) {
-    if (pc.kd == nullptr || pc.ld < spc2 + 1) return cudaErrorInvalidValue;
-    const long long total = (long long)n_pix * (spc2 + 1);
-    const int threads = 256;
+cudaError_t launch_pix_tables(const PixConst& pc, int m, int force, int n_pix, int spc2,
+                              cudaStream_t st) {
+    const int M = aff_modes(m), spc = spc2 / 2;
+    const bool rate = rate_law(force);
+    const int words = aff_row(M, rate);
+    if (pc.kd == nullptr || pc.ld < spc2 + 1 || pc.ld_rows < words * spc || pc.ld64 < 2 * spc)
+        return cudaErrorInvalidValue;
+    const long long total = (long long)n_pix * spc;
+    const int threads = 128;
     pix_tables_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, st>>>(
-        pc.kd, n_pix, spc2, pc.ld, const_cast<double*>(pc.tab64), const_cast<float*>(pc.tab32));
+        pc, n_pix, spc2, words, 2 + 2 * M + (rate ? 3 : 0),
+        const_cast<double*>(pc.tab64), const_cast<float*>(pc.tab32), const_cast<float*>(pc.rows));
     return cudaGetLastError();
 }
 

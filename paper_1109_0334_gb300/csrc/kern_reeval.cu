@@ -2,13 +2,13 @@
 // RK4 solution of Eq. 2, Sec. 3.2) by multiple shooting in time.
 //
 // FP64 arithmetic on this GPU issues at a small fraction of the FP32 rate,
-// so one thread stepping a whole record in FP64 needs ~7 us per RK4 step.
+// so one thread stepping a whole record in FP64 needs 5 to 7 us per RK4 step.
 // The record is instead cut into segments of AFM_SEG steps that are
 // integrated concurrently, one thread each, and the segment start states
 // are made consistent by Newton's method on the matching conditions
 // Z_{b+1} = Phi_b(Z_b), Phi_b being AFM_SEG FP64 RK4 steps:
-//   guess  one thread integrates the winner in FP32 (compensated, as the
-//          swarm kernels do) and keeps the state at every segment start;
+//   guess  one thread integrates the winner in FP32 (compensated, in the
+//          affine form) and keeps the state at every segment start;
 //   sweep  (twice) every segment is integrated in FP64 from its start Z_b,
 //          giving E_b = Phi_b(Z_b), while its tangent map J_b = dPhi_b/dZ_b
 //          is propagated in FP32 (the RK4 step linearised about the FP64
@@ -21,6 +21,10 @@
 // segment's end and the next segment's start exceeds 1e-9 (scaled units),
 // or anything is non-finite, the final kernel integrates the whole record
 // once more, sequentially, in FP64.
+//
+// A 25 600-step record (three modes, DMT): the affine step (afm_affine.cuh)
+// took 1.7 ms off the ~6 ms of guess and passes in the stage form; the guess,
+// one thread's 25 600 FP32 steps, is most of what is left.
 #include "afm_reeval.cuh"
 
 namespace afm {
@@ -64,8 +68,10 @@ __global__ void __launch_bounds__(256) reeval_guess_kernel(const KConst<float> K
                                                            const float* __restrict__ U) {
     extern __shared__ __align__(16) float tabf[];
     __shared__ double red[256];
-    build_drive_table(Kf, tabf);
-    build_drive_table(Kd, R.tab);
+    aff::build_rows<float, M, FORCE>(Kf, tabf);
+    const int spc = Kd.spc2 >> 1;
+    for (int j = threadIdx.x; j < spc; j += blockDim.x)
+        sincospi((2.0 / (double)spc) * (double)j, &R.tab[2 * j], &R.tab[2 * j + 1]);
     double acc = 0.0;
     const int nv = Kd.n_steps * (Kd.np > 0 ? Kd.np : 1);   // record values
     for (int n = threadIdx.x; n < nv; n += blockDim.x) acc += (double)U[n] * (double)U[n];
@@ -93,27 +99,7 @@ __global__ void __launch_bounds__(256) reeval_guess_kernel(const KConst<float> K
         Y[i] = Kd.q0[i];
         Y[M + i] = Kd.v0[i];
     }
-    float q[M], v[M], cq[M], cv[M];
-    init_state<float, M>(Kf, q, v, cq, cv);
-    int j = 0, b = 1, next = AFM_SEG;
-    const int n = Kf.n_steps, spc2 = Kf.spc2;
-    for (int s = 0; s < n; ++s) {
-        const float g0 = tabf[j], gh = tabf[j + 1], g1 = tabf[j + 2];
-        j += 2;
-        if (j >= spc2) j = 0;
-        rk4_step<float, M, FORCE>(Kf, c, q, v, cq, cv, g0, gh, g1);
-        if (s + 1 == next) {
-            if (b < R.B) {
-#pragma unroll
-                for (int i = 0; i < M; ++i) {
-                    Y[(size_t)b * S2 + i] = (double)q[i] - (double)cq[i];
-                    Y[(size_t)b * S2 + M + i] = (double)v[i] - (double)cv[i];
-                }
-            }
-            ++b;
-            next += AFM_SEG;
-        }
-    }
+    guess_starts<M, FORCE>(Kf, Kd, c, tabf, Kf.n_steps, R.B, Y);
 }
 
 // One thread per segment b: AFM_SEG FP64 steps from Z_b -> E_b and the
@@ -129,43 +115,37 @@ __global__ void __launch_bounds__(32) reeval_pass_kernel(const KConst<double> K,
     const int lane = threadIdx.x;
     const int b = blockIdx.x * 32 + lane;
     if (b >= R.B) return;
-    const Coef<double> c = winner_coef(*R.win);
+    const Coef<double> cw = winner_coef(*R.win);
+    const aff::LawCoef<double> c = aff::law_coef(cw);
     Coef<float> cf;
-    cf.c0 = (float)c.c0;
-    cf.c1 = (float)c.c1;
-    cf.c2 = (float)c.c2;
-    cf.c3 = (float)c.c3;
-    double q[M], v[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        q[i] = Z[(size_t)b * S2 + i];
-        v[i] = Z[(size_t)b * S2 + M + i];
-    }
+    cf.c0 = (float)cw.c0;
+    cf.c1 = (float)cw.c1;
+    cf.c2 = (float)cw.c2;
+    cf.c3 = (float)cw.c3;
+    aff::State<double, M, aff::NONE> st;
+    aff::import_state<M>(K, Z + (size_t)b * S2, Z + (size_t)b * S2 + M, st);
     const int n0 = b * AFM_SEG;
     const int n1 = min(n0 + AFM_SEG, K.n_steps);
-    int j = (int)((2ll * n0) % K.spc2);
+    const int spc = K.spc2 >> 1;
+    int j = n0 % spc;
     double S = 0.0;
     for (int s = n0; s < n1; ++s) {
-        const double g0 = R.tab[j], gh = R.tab[j + 1], g1 = R.tab[j + 2];
-        j += 2;
-        if (j >= K.spc2) j = 0;
-        step64<M, FORCE, TANGENT>(K, c, cf, q, v, g0, gh, g1, rec + lane + (s - n0) * kRec * 32);
+        double r[aff::Rows<M, FORCE>::words];
+        drive_terms<M, FORCE, true>(K, R.tab, j, r);
+        if (++j == spc) j = 0;
+        step64<M, FORCE, TANGENT>(K, c, cf, r, st, rec + lane + (s - n0) * kRec * 32);
         if (K.np > 0) {   // deflection points
             for (int k = 0; k < K.np; ++k) {
-                double uk = K.phi[k][0] * q[0];
-#pragma unroll
-                for (int i = 1; i < M; ++i) uk = fma(K.phi[k][i], q[i], uk);
-                const double r = (double)U[(size_t)s * K.np + k] - uk;
-                S = fma(r, r, S);
+                const double e = (double)U[(size_t)s * K.np + k] - aff::point_defl(K, k, st);
+                S = fma(e, e, S);
             }
         } else {
-            double u = q[0];
-#pragma unroll
-            for (int i = 1; i < M; ++i) u += q[i];
-            const double r = (double)U[s] - u;
-            S = fma(r, r, S);
+            const double e = (double)U[s] - aff::tip(st);
+            S = fma(e, e, S);
         }
     }
+    double q[M], v[M];
+    aff::export_state<double, M, aff::NONE>(K, st, q, v);
 #pragma unroll
     for (int i = 0; i < M; ++i) {
         R.E[(size_t)b * S2 + i] = q[i];
@@ -286,10 +266,7 @@ __global__ void __launch_bounds__(256) reeval_final_kernel(const KConst<double> 
     const double defect = rd[0];
     int segs = R.B;
     if (!(defect <= kDefectTol) || !isfinite(S64)) {
-        S64 = K.np > 0 ? integrate_points<double, M, FORCE, float>(K, winner_coef(w), R.tab, U,
-                                                                   nullptr, 0, 0, K.n_steps)
-                       : integrate<double, M, FORCE, float>(K, winner_coef(w), R.tab, U, nullptr,
-                                                            0, 0, K.n_steps);
+        S64 = integrate64<M, FORCE, true>(K, aff::law_coef(winner_coef(w)), R.tab, U, K.n_steps);
         segs = 0;
     }
     double th[AFM_MAXD];
@@ -371,9 +348,14 @@ cudaError_t launch_reeval(const KConst<float>& Kf, const KConst<double>& Kd, con
         return cudaErrorInvalidValue;
     return dispatch_m13(Kd.m, Kd.force, [&](auto Mc, auto Fc) -> cudaError_t {
         constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;
-        const size_t smem = sizeof(float) * (size_t)(Kf.spc2 + 1);
+        const size_t smem = aff_table_bytes<float, M, FORCE>(Kf.spc2);
+        cudaError_t e = cudaSuccess;
+        if (smem > 40 * 1024)
+            e = cudaFuncSetAttribute(reeval_guess_kernel<M, FORCE>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
         reeval_guess_kernel<M, FORCE><<<1, 256, smem, st>>>(Kf, Kd, R, U);
-        cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         const int grid = (R.B + 31) / 32;
         for (int k = 0; e == cudaSuccess && k < kSweeps; ++k) {
             reeval_pass_kernel<M, FORCE, true><<<grid, 32, 0, st>>>(Kd, R, R.start[k & 1], U);

@@ -12,6 +12,12 @@
 //            misfit share; one thread per slot adds its shares in order,
 //            checks the joins (sequential FP64 fallback past 1e-9) and fills
 //            the result record.
+// The passes are bound by FP64 issue (~150 FP64 instructions per step in the
+// affine form with one of reciprocal and square root per force, ~240 in the
+// stage form), the guess by one warp's instruction stream over the longest
+// record.  304 pixels of 5 120 to 15 360 steps: 3.0 ms less than in the stage
+// form, with each slot's sum of U^2 (a serial FP64 loop of the guess thread
+// before) taken by a warp.
 #include "afm_reeval.cuh"
 
 namespace afm {
@@ -49,7 +55,7 @@ __device__ __forceinline__ const KConst<T>& pix_k(const KConst<T>& K, const KCon
 template <bool PP>
 __device__ __forceinline__ const double* pix_tab64(const ReevalBatch& R, const BatchArgs& a, int pix) {
     if constexpr (PP)
-        return a.pix.tab64 + (size_t)pix * a.pix.ld;
+        return a.pix.tab64 + (size_t)pix * a.pix.ld64;
     else
         return R.tab;
 }
@@ -71,18 +77,17 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
                                                        const ReevalBatch R, const BatchArgs a) {
     extern __shared__ __align__(16) float tabs[];
     if constexpr (!PP) {
-        build_drive_table(Kf0, tabs);
-        if (blockIdx.x == 0) build_drive_table(Kd0, R.tab);
+        aff::build_rows<float, M, FORCE>(Kf0, tabs);
+        if (blockIdx.x == 0) aff::build_rows<double, M, FORCE>(Kd0, R.tab);
         __syncthreads();
     }
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n_pix) return;
+    const int i = blockIdx.x * 32 + threadIdx.x;   // warp 0's lanes; the others built the rows
+    if (threadIdx.x >= 32 || i >= a.n_pix) return;
     const int pix = slot_pixel(a, i);
     const KConst<float>& Kf = pix_k<PP>(Kf0, a.pix.kf, pix);
     const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
-    const float* tabf = PP ? a.pix.tab32 + (size_t)pix * a.pix.ld : tabs;
+    const float* tabf = PP ? a.pix.rows + (size_t)pix * a.pix.ld_rows : tabs;
     const int n = slot_steps(a, pix);
-    const float* U = a.U + a.off[pix];
     double xd[AFM_MAXD];
     for (int d = 0; d < AFM_MAXD; ++d) xd[d] = a.res[pix].x[d];
     const Coef<double> cd = make_coef<double, double>(Kd, xd);
@@ -90,9 +95,6 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
     R.coef[4 * (size_t)i + 1] = cd.c1;
     R.coef[4 * (size_t)i + 2] = cd.c2;
     R.coef[4 * (size_t)i + 3] = cd.c3;
-    double u2 = 0.0;
-    for (int s = 0; s < n; ++s) u2 = fma((double)U[s], (double)U[s], u2);
-    R.u2[i] = u2;
     const Coef<float> c = make_coef<float, double>(Kf, xd);
     constexpr int S2 = 2 * M;
     double* Y = R.Z + (size_t)i * R.maxB * S2;
@@ -102,28 +104,20 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
         Y[M + k] = Kd.v0[k];
     }
     const int B = slot_segments(R, n);
-    float q[M], v[M], cq[M], cv[M];
-    init_state<float, M>(Kf, q, v, cq, cv);
-    int j = 0, b = 1, next = AFM_SEG;
-    const int spc2 = Kf.spc2;
-    // the state after step (b * AFM_SEG) starts segment b; the last segment's
-    // start comes from step (B - 1) * AFM_SEG
-    const int n_guess = (B - 1) * AFM_SEG;
-    for (int s = 0; s < n_guess; ++s) {
-        const float g0 = tabf[j], gh = tabf[j + 1], g1 = tabf[j + 2];
-        j += 2;
-        if (j >= spc2) j = 0;
-        rk4_step<float, M, FORCE>(Kf, c, q, v, cq, cv, g0, gh, g1);
-        if (s + 1 == next) {
+    guess_starts<M, FORCE>(Kf, Kd, c, tabf, n, B, Y);
+}
+
+// Sum of U^2 of each slot's record, one warp per slot.
+__global__ void __launch_bounds__(128) rb_sumsq_kernel(const ReevalBatch R, const BatchArgs a) {
+    const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+    if (i >= a.n_pix) return;
+    const int pix = slot_pixel(a, i), n = slot_steps(a, pix);
+    const float* U = a.U + a.off[pix];
+    double u2 = 0.0;
+    for (int s = threadIdx.x & 31; s < n; s += 32) u2 = fma((double)U[s], (double)U[s], u2);
 #pragma unroll
-            for (int k = 0; k < M; ++k) {
-                Y[(size_t)b * S2 + k] = (double)q[k] - (double)cq[k];
-                Y[(size_t)b * S2 + M + k] = (double)v[k] - (double)cv[k];
-            }
-            ++b;
-            next += AFM_SEG;
-        }
-    }
+    for (int o = 16; o > 0; o >>= 1) u2 += __shfl_xor_sync(0xffffffffu, u2, o);
+    if ((threadIdx.x & 31) == 0) R.u2[i] = u2;
 }
 
 template <int M, int FORCE, bool TANGENT, bool PP>
@@ -141,34 +135,31 @@ __global__ void __launch_bounds__(32) rb_pass_kernel(const KConst<double> K0, co
     const KConst<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
     const double* tab = pix_tab64<PP>(R, a, pix);
     const float* U = a.U + a.off[pix];
-    const Coef<double> c = slot_coef(R, i);
+    const Coef<double> cw = slot_coef(R, i);
+    const aff::LawCoef<double> c = aff::law_coef(cw);
     Coef<float> cf;
-    cf.c0 = (float)c.c0;
-    cf.c1 = (float)c.c1;
-    cf.c2 = (float)c.c2;
-    cf.c3 = (float)c.c3;
+    cf.c0 = (float)cw.c0;
+    cf.c1 = (float)cw.c1;
+    cf.c2 = (float)cw.c2;
+    cf.c3 = (float)cw.c3;
     const size_t g = (size_t)i * R.maxB + b;   // global segment index
-    double q[M], v[M];
-#pragma unroll
-    for (int k = 0; k < M; ++k) {
-        q[k] = R.Z[g * S2 + k];
-        v[k] = R.Z[g * S2 + M + k];
-    }
+    aff::State<double, M, aff::NONE> st;
+    aff::import_state<M>(K, R.Z + g * S2, R.Z + g * S2 + M, st);
     const int n0 = b * AFM_SEG;
     const int n1 = min(n0 + AFM_SEG, n);
-    int j = (int)((2ll * n0) % K.spc2);
+    const int spc = K.spc2 >> 1;
+    int j = n0 % spc;
     double S = 0.0;
     for (int s = n0; s < n1; ++s) {
-        const double g0 = tab[j], gh = tab[j + 1], g1 = tab[j + 2];
-        j += 2;
-        if (j >= K.spc2) j = 0;
-        step64<M, FORCE, TANGENT>(K, c, cf, q, v, g0, gh, g1, rec + lane + (s - n0) * kRec * 32);
-        double u = q[0];
-#pragma unroll
-        for (int k = 1; k < M; ++k) u += q[k];
-        const double r = (double)U[s] - u;
-        S = fma(r, r, S);
+        double r[aff::Rows<M, FORCE>::words];
+        drive_terms<M, FORCE, PP || aff::Table<double, M, FORCE>::compact>(K, tab, j, r);
+        if (++j == spc) j = 0;
+        step64<M, FORCE, TANGENT>(K, c, cf, r, st, rec + lane + (s - n0) * kRec * 32);
+        const double e = (double)U[s] - aff::tip(st);
+        S = fma(e, e, S);
     }
+    double q[M], v[M];
+    aff::export_state<double, M, aff::NONE>(K, st, q, v);
 #pragma unroll
     for (int k = 0; k < M; ++k) {
         R.E[g * S2 + k] = q[k];
@@ -279,8 +270,8 @@ __global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, 
     }
     int segs = B;
     if (!(defect <= kDefectTol) || !isfinite(S64)) {
-        S64 = integrate<double, M, FORCE, float>(K, slot_coef(R, i), pix_tab64<PP>(R, a, pix),
-                                                 a.U + a.off[pix], nullptr, 0, 0, n);
+        S64 = integrate64<M, FORCE, PP || aff::Table<double, M, FORCE>::compact>(
+            K, aff::law_coef(slot_coef(R, i)), pix_tab64<PP>(R, a, pix), a.U + a.off[pix], n);
         segs = 0;
     }
     afm_result* r = a.res + pix;
@@ -304,22 +295,23 @@ __global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, 
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-size_t reeval_batch_bytes(int m, int n_steps, int spc, int n_pix) {
+size_t reeval_batch_bytes(int m, int force, int n_steps, int spc, int n_pix) {
     const size_t B = (size_t)reeval_segments(n_steps), S2 = 2 * (size_t)reeval_modes(m);
     const size_t segs = B * (size_t)n_pix;
-    return a256(sizeof(double) * 4 * (size_t)n_pix) + a256(sizeof(double) * (2 * (size_t)spc + 1)) +
+    return a256(sizeof(double) * 4 * (size_t)n_pix) + a256(sizeof(double) * (size_t)spc * aff_row64(reeval_modes(m), rate_law(force))) +
            a256(sizeof(double) * segs * S2) * 2 + a256(sizeof(float) * segs * S2 * S2) +
            a256(sizeof(double) * segs) + a256(sizeof(double) * (size_t)n_pix) + 256;
 }
 
-void reeval_batch_carve(void* base, int m, int n_steps, int spc, int n_pix, ReevalBatch* R) {
+void reeval_batch_carve(void* base, int m, int force, int n_steps, int spc, int n_pix,
+                        ReevalBatch* R) {
     const size_t B = (size_t)reeval_segments(n_steps), S2 = 2 * (size_t)reeval_modes(m);
     const size_t segs = B * (size_t)n_pix;
     char* p = static_cast<char*>(base);
     R->coef = reinterpret_cast<double*>(p);
     p += a256(sizeof(double) * 4 * (size_t)n_pix);
     R->tab = reinterpret_cast<double*>(p);
-    p += a256(sizeof(double) * (2 * (size_t)spc + 1));
+    p += a256(sizeof(double) * (size_t)spc * aff_row64(reeval_modes(m), rate_law(force)));
     R->Z = reinterpret_cast<double*>(p);
     p += a256(sizeof(double) * segs * S2);
     R->E = reinterpret_cast<double*>(p);
@@ -340,12 +332,21 @@ cudaError_t launch_reeval_batch(const KConst<float>& Kf, const KConst<double>& K
         constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;
         auto run = [&](auto Pc) -> cudaError_t {
             constexpr bool PP = decltype(Pc)::value;
-            const size_t smem = PP ? 0 : sizeof(float) * (size_t)(Kf.spc2 + 1);
-            rb_guess_kernel<M, FORCE, PP><<<(a.n_pix + 127) / 128, 128, smem, st>>>(Kf, Kd, R, a);
-            cudaError_t e = cudaGetLastError();
+            const size_t smem = PP ? 0 : aff_table_bytes<float, M, FORCE>(Kf.spc2);
+            cudaError_t e = cudaSuccess;
+            if (smem > 48 * 1024)
+                e = cudaFuncSetAttribute(rb_guess_kernel<M, FORCE, PP>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            // 32 slots per block: each warp on an SM of its own for as long as
+            // there are SMs (the longest record's warp sets the time)
+            rb_guess_kernel<M, FORCE, PP><<<(a.n_pix + 31) / 32, 128, smem, st>>>(Kf, Kd, R, a);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
             const long long segs = (long long)a.n_pix * R.maxB;
             const int grid = (int)((segs + 31) / 32);
             const int cgrid = (a.n_pix * 32 + 127) / 128;
+            rb_sumsq_kernel<<<cgrid, 128, 0, st>>>(R, a);
+            e = cudaGetLastError();
             for (int k = 0; e == cudaSuccess && k < kSweeps; ++k) {
                 rb_pass_kernel<M, FORCE, true, PP><<<grid, 32, 0, st>>>(Kd, R, a);
                 if ((e = cudaGetLastError()) != cudaSuccess) break;
