@@ -173,27 +173,14 @@ typedef struct afm_ctx afm_ctx;
 afm_status afm_ctx_create(int device, afm_ctx** out);
 afm_status afm_ctx_destroy(afm_ctx* ctx);
 
-/* Lanes per particle of the fused inversion iteration (afm_invert,
- * afm_invert_polished, deflection-point records included).  For
- * afm_forward_batch, AFM_LANES_ONE also keeps one particle per thread where
- * large FP32 DMT batches (1 or 3 modes, P >= 65536) otherwise run two
- * particles per thread in paired FP32 instructions (bit-identical).
- * A swarm too small to fill the GPU is latency-bound
- * along each particle's RK4 recurrence (Sec. 3.2); spreading a particle over
- * several lanes of a warp shortens the chain.  Every variant is bit-identical
- * to the one-lane arithmetic; a variant the problem does not support runs
- * the automatic choice.
- *   AFM_LANES_AUTO    the library's choice (default)
- *   AFM_LANES_ONE     one lane per particle
- *   AFM_LANES_STAGES  two lanes, the tip forces of RK4 stages 1/3 and 2/4
- *                     evaluated by one lane each (rate-free force laws,
- *                     1 or 3 modes, P <= 9728)
- *   AFM_LANES_MODES2  two lanes, the modes split between them (rate-free
- *                     laws, 2 or 3 modes, P <= 9728)
- *   AFM_LANES_MODES4  four lanes, one mode each (rate-free laws, 2 or 3
- *                     modes, P <= 4864)
- *   AFM_LANES_MODES3  three lanes, one mode each, ten particles per warp
- *                     (rate-free laws, 2 or 3 modes, P <= 6080)
+/* Particle layout.  For afm_forward_batch, AFM_LANES_ONE keeps one particle
+ * per thread where large FP32 DMT batches (1 or 3 modes, P >= 65536) otherwise
+ * run two particles per thread in paired FP32 instructions (bit-identical).
+ * The fused inversion iteration (afm_invert, afm_invert_polished,
+ * deflection-point records included) runs one lane per particle whatever the
+ * value: it is faster than the layouts that spread a particle's modes or
+ * stage forces over several lanes, whose values are still accepted
+ * (bit-identical results).
  * Returns AFM_ERR_INVALID_ARG for an unknown value. */
 typedef enum {
     AFM_LANES_AUTO = 0,

@@ -185,23 +185,9 @@ cudaError_t launch_pso_move(const PsoConst& pc, const SwarmPtrs& sw, int it, cud
 // the move with a given global-best position gb [D] (a slice of a split swarm)
 cudaError_t launch_pso_move_given(const PsoConst& pc, const SwarmPtrs& sw, const float* gb, int it,
                                   cudaStream_t st);
-// fused inversion iteration (it = 0: initial evaluation); `lanes` picks the
-// lanes-per-particle variant (afm_lanes of afminv.h; all are bit-identical,
-// a variant the problem does not support runs the automatic choice)
+// fused inversion iteration (it = 0: initial evaluation)
 cudaError_t launch_invert_iter(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
-                               const float* U, float* history, int it, cudaStream_t st,
-                               int lanes = 0);
-// the same iteration with two lanes per particle, the RK4 stage forces split
-// between them (rate-free laws, 1 or 3 modes, P <= 9728)
-bool pair_supported(int m, int force, int P);
-cudaError_t launch_invert_pair(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
                                const float* U, float* history, int it, cudaStream_t st);
-// the same iteration with the modes of a particle spread over 2 or 4 lanes
-// (rate-free laws, 2 or 3 modes, P <= 19456 / lanes)
-bool modes_supported(int m, int force, int P, int lanes);
-cudaError_t launch_invert_modes(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
-                                const float* U, float* history, int it, int lanes,
-                                cudaStream_t st);
 // base-motion inversion (drive_mode 1, kern_drive.cu)
 cudaError_t launch_forward_drive_f32(const KConst<float>& K, const float* x, int P, float* defl,
                                      const float* U, float* S, cudaStream_t st);
@@ -216,17 +202,8 @@ cudaError_t launch_forward_points_f32(const KConst<float>& K, const float* x, in
                                       const float* U, float* S, cudaStream_t st);
 cudaError_t launch_forward_points_f64(const KConst<double>& K, const double* x, int P, double* defl,
                                       const double* U, double* S, cudaStream_t st);
-// (lanes: AFM_LANES_ONE runs one lane per particle, any other value one
-// mode per lane where points_modes_supported; bit-identical)
 cudaError_t launch_invert_points(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
-                                 const float* U, float* history, int it, cudaStream_t st,
-                                 int lanes = 0);
-// the points iteration with one mode per lane (rate-free laws, 2 or 3
-// modes, lanes = modes, P <= 19456 / modes)
-bool points_modes_supported(int m, int force, int P, int np);
-cudaError_t launch_invert_points_modes(const KConst<float>& K, const PsoConst& pc,
-                                       const SwarmPtrs& sw, const float* U, float* history, int it,
-                                       cudaStream_t st);
+                                 const float* U, float* history, int it, cudaStream_t st);
 cudaError_t launch_points_final(const KConst<double>& K, const PsoConst& pc, const SwarmPtrs& sw,
                                 const float* U, float* history, void* result, cudaStream_t st);
 // winner re-evaluation in FP64 and result record

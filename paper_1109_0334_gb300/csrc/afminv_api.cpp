@@ -45,7 +45,7 @@ struct afm_ctx {
     std::vector<afm_batch_graph> batch_graphs;
     // kernel timing (afm_profile_*): events around each fused iteration launch
     bool profiling = false;
-    // lanes per particle of the fused inversion iteration (afm_lanes)
+    // particle layout of afm_forward_batch (afm_lanes)
     int lanes = AFM_LANES_AUTO;
     std::vector<cudaEvent_t> ev_pool;   // reusable events
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending;
@@ -1060,7 +1060,7 @@ cudaError_t invert_iter_timed(afm_ctx* ctx, const KConst<float>& K, const PsoCon
                               const SwarmPtrs& sw, const float* U, float* history, int it,
                               cudaStream_t s) {
     return timed_launch(ctx, s, [&] {
-        return afm::launch_invert_iter(K, pc, sw, U, history, it, s, ctx->lanes);
+        return afm::launch_invert_iter(K, pc, sw, U, history, it, s);
     });
 }
 
@@ -1450,9 +1450,8 @@ afm_status afm_invert(afm_ctx* ctx, const afm_problem* prob, const float* U,
     }
     for (int it = 0; it <= cfg->iters; ++it)
         AFM_CUDA(timed_launch(ctx, s, [&] {
-                     return prob->n_points > 0 ? afm::launch_invert_points(Kf, pc, sw, U, history, it, s, ctx->lanes)
-                                               : afm::launch_invert_iter(Kf, pc, sw, U, history, it, s,
-                                                                         ctx->lanes);
+                     return prob->n_points > 0 ? afm::launch_invert_points(Kf, pc, sw, U, history, it, s)
+                                               : afm::launch_invert_iter(Kf, pc, sw, U, history, it, s);
                  }),
                  "invert iteration kernel");
     if (reeval_extra(*prob) > 0) {
@@ -1736,7 +1735,7 @@ afm_status afm_invert_polished(afm_ctx* ctx, const afm_problem* prob, const floa
     AFM_CUDA(afm::launch_pso_init(pc, sw, s), "pso init kernel");
     for (int it = 0; it <= cfg->iters; ++it)
         AFM_CUDA(timed_launch(ctx, s, [&] {
-                     return afm::launch_invert_iter(Kf, pc, sw, U, history, it, s, ctx->lanes);
+                     return afm::launch_invert_iter(Kf, pc, sw, U, history, it, s);
                  }),
                  "invert iteration kernel");
     const int fin = (cfg->iters + 1) & 1;

@@ -9,6 +9,7 @@
 #include "afm_device.cuh"
 #include "afm_f32x2.cuh"
 #include "afm_launch.h"
+#include "afm_warp.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -51,6 +52,36 @@ __global__ void fwd_kernel(const KConst<T> K, const T* __restrict__ x, int P,
     if (S != nullptr) {
         if (!(s < (T)INFINITY)) {
             s = (T)INFINITY;
+            if (flags != nullptr) atomicAdd(flags, 1);
+        }
+        S[p] = s;
+    }
+}
+
+// The FP32 solve for batches of at most one warp per SM sub-partition: one
+// particle per lane (integrate_warp;
+// bit-identical to fwd_kernel).  The first ppb threads of a block carry
+// particles; all of them build the drive table.
+template <int M, int FORCE>
+__global__ void __launch_bounds__(128, 1)
+fwd_warp_kernel(const KConst<float> K, const float* __restrict__ x, int P, int ppb,
+                float* __restrict__ defl, const float* __restrict__ U, float* __restrict__ S,
+                int* __restrict__ flags) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* tab = reinterpret_cast<float*>(smem_raw);
+    build_drive_table(K, tab);
+    __syncthreads();
+    const int p0 = blockIdx.x * ppb + threadIdx.x;
+    if ((int)(threadIdx.x & ~31u) >= ppb || (p0 & ~31) >= P) return;   // whole warps
+    const bool store = p0 < P;
+    const int p = min(p0, P - 1);
+    float xd[AFM_MAXD];
+    for (int d = 0; d < K.D; ++d) xd[d] = x[(size_t)d * P + p];
+    const Coef<float> c = make_coef<float, float>(K, xd);
+    float s = integrate_warp<M, FORCE>(K, c, tab, U, defl, P, p, K.n_steps, store);
+    if (S != nullptr && store) {
+        if (!(s < INFINITY)) {
+            s = INFINITY;
             if (flags != nullptr) atomicAdd(flags, 1);
         }
         S[p] = s;
@@ -142,6 +173,15 @@ cudaError_t launch_forward_f32(const KConst<float>& K, const float* x, int P, fl
                                const float* U, float* S, int* flags, cudaStream_t st, int lanes) {
     if (forward_x2_ok(K.m, K.force, P, lanes))
         return launch_forward_x2(K, x, P, defl, U, S, flags, st);
+    if (P <= warp::max_particles()) {
+        const int ppb = warp::per_block(P);
+        const size_t smem = sizeof(float) * (size_t)(K.spc2 + 1);
+        return warp::dispatch(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
+            fwd_warp_kernel<decltype(Mc)::value, decltype(Fc)::value>
+                <<<(P + ppb - 1) / ppb, 128, smem, st>>>(K, x, P, ppb, defl, U, S, flags);
+            return cudaGetLastError();
+        });
+    }
     return launch_forward<float>(K, x, P, defl, U, S, flags, st);
 }
 

@@ -9,6 +9,7 @@
 #include "../../include/afminv.h"
 #include "afm_device.cuh"
 #include "afm_launch.h"
+#include "afm_warp.cuh"
 
 namespace afm {
 
@@ -172,85 +173,113 @@ cudaError_t launch_pso_move(const PsoConst& pc, const SwarmPtrs& sw, int it, cud
 // Personal-best positions and the global-best key are double-buffered by
 // iteration parity so that no launch reads what it writes.
 // ---------------------------------------------------------------------------
+// Bests of one particle after its evaluation (misfit s at x); returns its
+// global-best key.
+__device__ __forceinline__ unsigned long long update_best(const PsoConst& pc, const SwarmPtrs& sw,
+                                                          const float* x, float s, int p, int it) {
+    const int rd = it & 1, wr = (it + 1) & 1;
+    s = sanitize_misfit(s, sw.flags);
+    float best = sw.pbS[p];
+    const bool improved = s < best || it == 0;
+    if (s < best) best = s;
+    sw.pbS[p] = best;
+    for (int d = 0; d < pc.D; ++d)
+        sw.pb[wr][(size_t)d * pc.P + p] = improved ? x[d] : sw.pb[rd][(size_t)d * pc.P + p];
+    return best_key(best, p);
+}
+
+// Loads particle p and, from the second iteration on, moves it (Eq. 8).
+// store: write the moved particle back.
+__device__ __forceinline__ void load_moved(const PsoConst& pc, const SwarmPtrs& sw, float* x, int p,
+                                           int it, bool store) {
+    const int rd = it & 1;
+    float v[AFM_MAXD];
+    for (int d = 0; d < pc.D; ++d) {
+        x[d] = sw.x[(size_t)d * pc.P + p];
+        v[d] = sw.v[(size_t)d * pc.P + p];
+    }
+    if (it == 0) return;
+    const int g = min((int)(*sw.gkey[rd] & 0x7fffffffu), pc.P - 1);
+    float pb[AFM_MAXD], gb[AFM_MAXD];
+    for (int d = 0; d < pc.D; ++d) {
+        pb[d] = sw.pb[rd][(size_t)d * pc.P + p];
+        gb[d] = sw.pb[rd][(size_t)d * pc.P + g];
+    }
+    pso_move_dev(pc, x, v, pb, gb, p, it);
+    // lanes past the swarm repeat its last particle: its owner writes only
+    // after every lane of the warp has read
+    __syncwarp();
+    if (!store) return;
+    for (int d = 0; d < pc.D; ++d) {
+        sw.x[(size_t)d * pc.P + p] = x[d];
+        sw.v[(size_t)d * pc.P + p] = v[d];
+    }
+}
+
+// One particle per lane, up to one warp per SM sub-partition
+// (integrate_warp, afm_warp.cuh): 1024 particles x 25 600 steps, three modes,
+// DMT: 2.55 ms a launch, 3.87 ms with one mode per lane.
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128, 1)
 invert_iter_kernel(const KConst<float> K, const PsoConst pc, SwarmPtrs sw,
+                   const float* __restrict__ U, float* __restrict__ history, int it, int ppb) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* tab = reinterpret_cast<float*>(smem_raw);
+    build_drive_table(K, tab);
+    __syncthreads();
+    const int p0 = blockIdx.x * ppb + threadIdx.x;
+    if ((int)(threadIdx.x & ~31u) >= ppb || (p0 & ~31) >= pc.P) return;   // whole warps
+    const bool store = p0 < pc.P;
+    const int p = min(p0, pc.P - 1);
+    if (it > 0 && p0 == 0 && history != nullptr)
+        history[it - 1] = __uint_as_float((uint32_t)(*sw.gkey[it & 1] >> 32));
+    float x[AFM_MAXD];
+    load_moved(pc, sw, x, p, it, store);
+    const Coef<float> c = make_coef<float, float>(K, x);
+    const float s = integrate_warp<M, FORCE>(K, c, tab, U, nullptr, 0, p, K.n_steps, false);
+    const unsigned long long key = store ? update_best(pc, sw, x, s, p, it) : ~0ull;
+    warp_min_atomic(key, sw.gkey[(it + 1) & 1]);
+}
+
+// Larger swarms: several warps per sub-partition hide each other's latency.
+template <int M, int FORCE>
+__global__ void __launch_bounds__(128)
+invert_wide_kernel(const KConst<float> K, const PsoConst pc, SwarmPtrs sw,
                    const float* __restrict__ U, float* __restrict__ history, int it) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* tab = reinterpret_cast<float*>(smem_raw);
     build_drive_table(K, tab);
     __syncthreads();
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int rd = it & 1, wr = (it + 1) & 1;
-    const float* pb_rd = sw.pb[rd];
-    float* pb_wr = sw.pb[wr];
+    const int p0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool store = p0 < pc.P;
+    const int p = min(p0, pc.P - 1);
+    if (it > 0 && p0 == 0 && history != nullptr)
+        history[it - 1] = __uint_as_float((uint32_t)(*sw.gkey[it & 1] >> 32));
+    float x[AFM_MAXD];
+    load_moved(pc, sw, x, p, it, store);
     unsigned long long key = ~0ull;
-    if (it > 0 && p == 0 && history != nullptr)
-        history[it - 1] = __uint_as_float((uint32_t)(*sw.gkey[rd] >> 32));
-    if (p < pc.P) {
-        float x[AFM_MAXD], v[AFM_MAXD];
-        for (int d = 0; d < pc.D; ++d) {
-            x[d] = sw.x[(size_t)d * pc.P + p];
-            v[d] = sw.v[(size_t)d * pc.P + p];
-        }
-        if (it > 0) {
-            const int g = min((int)(*sw.gkey[rd] & 0x7fffffffu), pc.P - 1);
-            float pb[AFM_MAXD], gb[AFM_MAXD];
-            for (int d = 0; d < pc.D; ++d) {
-                pb[d] = pb_rd[(size_t)d * pc.P + p];
-                gb[d] = pb_rd[(size_t)d * pc.P + g];
-            }
-            pso_move_dev(pc, x, v, pb, gb, p, it);
-            for (int d = 0; d < pc.D; ++d) {
-                sw.x[(size_t)d * pc.P + p] = x[d];
-                sw.v[(size_t)d * pc.P + p] = v[d];
-            }
-        }
-        Coef<float> c = make_coef<float, float>(K, x);
-        float s = integrate<float, M, FORCE>(K, c, tab, U, nullptr, 0, p, K.n_steps);
-        s = sanitize_misfit(s, sw.flags);
-        float best = sw.pbS[p];
-        const bool improved = s < best || it == 0;
-        if (s < best) best = s;
-        sw.pbS[p] = best;
-        for (int d = 0; d < pc.D; ++d)
-            pb_wr[(size_t)d * pc.P + p] = improved ? x[d] : pb_rd[(size_t)d * pc.P + p];
-        key = best_key(best, p);
+    if (store) {
+        const Coef<float> c = make_coef<float, float>(K, x);
+        const float s = integrate<float, M, FORCE>(K, c, tab, U, nullptr, 0, p, K.n_steps);
+        key = update_best(pc, sw, x, s, p, it);
     }
-    warp_min_atomic(key, sw.gkey[wr]);
+    warp_min_atomic(key, sw.gkey[(it + 1) & 1]);
 }
 
 cudaError_t launch_invert_iter(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
-                               const float* U, float* history, int it, cudaStream_t st,
-                               int lanes) {
-    // small swarms of rate-free force laws: several lanes per particle
-    // (kern_modes.cu: modes split; kern_pair.cu: RK4 stage forces split).
-    // Automatic choice, by measurement on the 3-mode DMT swarm of 1024
-    // particles (per launch: one lane 4.59 ms, stages 4.53, modes over 4
-    // lanes 4.41, over 2 lanes 4.30, over 3 lanes 3.66): one mode per lane
-    // for 3 modes, modes over 2 lanes for 2, else stages.
-    const bool m2 = modes_supported(K.m, K.force, pc.P, 2);
-    const bool m4 = modes_supported(K.m, K.force, pc.P, 4);
-    const bool m3 = modes_supported(K.m, K.force, pc.P, 3);
-    const bool st2 = pair_supported(K.m, K.force, pc.P);
-    const bool ok = lanes == AFM_LANES_ONE || (lanes == AFM_LANES_STAGES && st2) ||
-                    (lanes == AFM_LANES_MODES2 && m2) || (lanes == AFM_LANES_MODES4 && m4) ||
-                    (lanes == AFM_LANES_MODES3 && m3);
-    if (!ok)
-        lanes = (K.m == 3 && m3) ? AFM_LANES_MODES3
-                : m2             ? AFM_LANES_MODES2
-                : st2            ? AFM_LANES_STAGES
-                                 : AFM_LANES_ONE;
-    if (lanes == AFM_LANES_MODES2) return launch_invert_modes(K, pc, sw, U, history, it, 2, st);
-    if (lanes == AFM_LANES_MODES4) return launch_invert_modes(K, pc, sw, U, history, it, 4, st);
-    if (lanes == AFM_LANES_MODES3) return launch_invert_modes(K, pc, sw, U, history, it, 3, st);
-    if (lanes == AFM_LANES_STAGES) return launch_invert_pair(K, pc, sw, U, history, it, st);
-    const int threads = pc.P <= 152 * 32 * 4 ? 32 : 128;
-    const int blocks = (pc.P + threads - 1) / threads;
+                               const float* U, float* history, int it, cudaStream_t st) {
     const size_t smem = sizeof(float) * (size_t)(K.spc2 + 1);
+    if (pc.P <= warp::max_particles()) {
+        const int ppb = warp::per_block(pc.P);
+        return warp::dispatch(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
+            invert_iter_kernel<decltype(Mc)::value, decltype(Fc)::value>
+                <<<(pc.P + ppb - 1) / ppb, 128, smem, st>>>(K, pc, sw, U, history, it, ppb);
+            return cudaGetLastError();
+        });
+    }
     return dispatch_mf(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
-        constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;
-        invert_iter_kernel<M, FORCE><<<blocks, threads, smem, st>>>(K, pc, sw, U, history, it);
+        invert_wide_kernel<decltype(Mc)::value, decltype(Fc)::value>
+            <<<(pc.P + 127) / 128, 128, smem, st>>>(K, pc, sw, U, history, it);
         return cudaGetLastError();
     });
 }

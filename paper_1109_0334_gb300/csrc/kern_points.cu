@@ -8,6 +8,7 @@
 
 #include "afm_device.cuh"
 #include "afm_launch.h"
+#include "afm_warp.cuh"
 
 namespace afm {
 
@@ -57,12 +58,13 @@ __global__ void fwd_points_kernel(const KConst<T> K, const T* __restrict__ x, in
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128, 1)
 invert_points_kernel(const KConst<float> K, const PsoConst pc, SwarmPtrs sw,
-                     const float* __restrict__ U, float* __restrict__ history, int it) {
+                     const float* __restrict__ U, float* __restrict__ history, int it, int ppb) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* tab = reinterpret_cast<float*>(smem_raw);
     build_drive_table(K, tab);
     __syncthreads();
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if ((int)(threadIdx.x & ~31u) >= ppb) return;   // whole warps
+    const int p = blockIdx.x * ppb + threadIdx.x;
     const int rd = it & 1, wr = (it + 1) & 1;
     const float* pb_rd = sw.pb[rd];
     float* pb_wr = sw.pb[wr];
@@ -89,7 +91,7 @@ invert_points_kernel(const KConst<float> K, const PsoConst pc, SwarmPtrs sw,
             }
         }
         const Coef<float> c = make_coef<float, float>(K, x);
-        float s = integrate_points<float, M, FORCE>(K, c, tab, U, nullptr, 0, p, K.n_steps);
+        float s = integrate_points_warp<M, FORCE>(K, c, tab, U, K.n_steps);
         if (!(s < INFINITY)) {
             if (sw.flags) atomicAdd(sw.flags, 1);
             s = INFINITY;
@@ -191,18 +193,12 @@ cudaError_t launch_forward_points_f64(const KConst<double>& K, const double* x, 
 }
 
 cudaError_t launch_invert_points(const KConst<float>& K, const PsoConst& pc, const SwarmPtrs& sw,
-                                 const float* U, float* history, int it, cudaStream_t st,
-                                 int lanes) {
-    // one mode per lane (kern_modes.cu) unless one lane is asked for; per
-    // launch on the three-point, 3-mode DMT swarm of 512 particles over
-    // 10240 steps: one lane 2.30 ms, one mode per lane 2.22 ms
-    if (lanes != AFM_LANES_ONE && points_modes_supported(K.m, K.force, pc.P, K.np))
-        return launch_invert_points_modes(K, pc, sw, U, history, it, st);
-    const int threads = pc.P <= 152 * 32 * 4 ? 32 : 128;
+                                 const float* U, float* history, int it, cudaStream_t st) {
     const size_t smem = sizeof(float) * (size_t)(K.spc2 + 1);
-    return dispatch_mf(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
+    const int ppb = warp::per_block(pc.P);
+    return warp::dispatch(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
         invert_points_kernel<decltype(Mc)::value, decltype(Fc)::value>
-            <<<(pc.P + threads - 1) / threads, threads, smem, st>>>(K, pc, sw, U, history, it);
+            <<<(pc.P + ppb - 1) / ppb, 128, smem, st>>>(K, pc, sw, U, history, it, ppb);
         return cudaGetLastError();
     });
 }
