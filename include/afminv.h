@@ -319,7 +319,9 @@ afm_status afm_adjoint(afm_ctx* ctx, const afm_problem* prob, const float* x, in
  * to afm_forward_batch), and the normal equations of the misfit Eq. 5,
  * H [P][D][D] = sum_n a_n a_n^T and b [P][D] = sum_n a_n (U_n - u_n), with
  * a_n = du_n/dx the tangent-linear sensitivities of the FP32 RK4 recurrence
- * (Eq. 2, Sec. 3.2) accumulated in FP32 blocks of 32 steps and FP64 totals.
+ * (Eq. 2, Sec. 3.2) accumulated in FP32 blocks of 32 steps and FP64 totals
+ * (along the force law's coefficients, mapped to x in FP64, where the free
+ * parameters are at least as many).
  * -2 b is the misfit gradient (as afm_adjoint's dS_dx); 2 H is the
  * Gauss-Newton Hessian.  H and b are device FP64 arrays. */
 afm_status afm_normal_equations(afm_ctx* ctx, const afm_problem* prob, const float* x, int P,

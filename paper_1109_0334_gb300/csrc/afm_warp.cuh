@@ -123,10 +123,15 @@ __device__ __forceinline__ void accel(const Modes<M>& C, const float* q, const f
     }
 }
 
-// One step (rk4_step); gh, g1: drive at t + h/2 and t + h.
+// Gaps and gap rates of a step's four stages.
+struct Gaps {
+    float d[4], r[4];
+};
+
+// One step (rk4_step); gh, g1: drive at t + h/2 and t + h; g: its stage gaps.
 template <int M, int FORCE>
 __device__ __forceinline__ void step(const Modes<M>& C, const Coef<float>& c, float gh, float g1,
-                                     State<M>& s) {
+                                     State<M>& s, Gaps& g) {
     float ggh[M], gg1[M], q2[M], q3[M], q4[M], v2[M], v3[M], v4[M], a1[M], a2[M], a3[M], a4[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -135,32 +140,45 @@ __device__ __forceinline__ void step(const Modes<M>& C, const Coef<float>& c, fl
     }
     axpy<M>(3.f, s.v, s.q, q2);
     if constexpr (!UsesRate<FORCE>::value) {
-        const float F2 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q2)), 0.f);
-        const float F1 = law<FORCE>(c, __fadd_rn(C.Zc, s.u), 0.f);
+        g.r[0] = g.r[1] = g.r[2] = g.r[3] = 0.f;
+        g.d[1] = __fadd_rn(C.Zc, sum<M>(q2));
+        g.d[0] = __fadd_rn(C.Zc, s.u);
+        const float F2 = law<FORCE>(c, g.d[1], 0.f);
+        const float F1 = law<FORCE>(c, g.d[0], 0.f);
         accel<M>(C, s.q, s.v, s.gg, F1, a1);
         axpy<M>(3.f, a1, s.v, v2);
         accel<M>(C, q2, v2, ggh, F2, a2);
         axpy<M>(3.f, v2, s.q, q3);
         axpy<M>(3.f, a2, s.v, v3);
         axpy<M>(6.f, v3, s.q, q4);
-        const float F4 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q4)), 0.f);
-        const float F3 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q3)), 0.f);
+        g.d[3] = __fadd_rn(C.Zc, sum<M>(q4));
+        g.d[2] = __fadd_rn(C.Zc, sum<M>(q3));
+        const float F4 = law<FORCE>(c, g.d[3], 0.f);
+        const float F3 = law<FORCE>(c, g.d[2], 0.f);
         accel<M>(C, q3, v3, ggh, F3, a3);
         axpy<M>(6.f, a3, s.v, v4);
         accel<M>(C, q4, v4, gg1, F4, a4);
     } else {
-        const float F1 = law<FORCE>(c, __fadd_rn(C.Zc, s.u), sum<M>(s.v));
+        g.d[0] = __fadd_rn(C.Zc, s.u);
+        g.r[0] = sum<M>(s.v);
+        const float F1 = law<FORCE>(c, g.d[0], g.r[0]);
         accel<M>(C, s.q, s.v, s.gg, F1, a1);
         axpy<M>(3.f, a1, s.v, v2);
-        const float F2 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q2)), sum<M>(v2));
+        g.d[1] = __fadd_rn(C.Zc, sum<M>(q2));
+        g.r[1] = sum<M>(v2);
+        const float F2 = law<FORCE>(c, g.d[1], g.r[1]);
         accel<M>(C, q2, v2, ggh, F2, a2);
         axpy<M>(3.f, v2, s.q, q3);
         axpy<M>(3.f, a2, s.v, v3);
-        const float F3 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q3)), sum<M>(v3));
+        g.d[2] = __fadd_rn(C.Zc, sum<M>(q3));
+        g.r[2] = sum<M>(v3);
+        const float F3 = law<FORCE>(c, g.d[2], g.r[2]);
         accel<M>(C, q3, v3, ggh, F3, a3);
         axpy<M>(6.f, v3, s.q, q4);
         axpy<M>(6.f, a3, s.v, v4);
-        const float F4 = law<FORCE>(c, __fadd_rn(C.Zc, sum<M>(q4)), sum<M>(v4));
+        g.d[3] = __fadd_rn(C.Zc, sum<M>(q4));
+        g.r[3] = sum<M>(v4);
+        const float F4 = law<FORCE>(c, g.d[3], g.r[3]);
         accel<M>(C, q4, v4, gg1, F4, a4);
     }
 #pragma unroll
@@ -173,6 +191,13 @@ __device__ __forceinline__ void step(const Modes<M>& C, const Coef<float>& c, fl
         s.gg[i] = gg1[i];
     }
     s.u = sum<M>(s.q);
+}
+
+template <int M, int FORCE>
+__device__ __forceinline__ void step(const Modes<M>& C, const Coef<float>& c, float gh, float g1,
+                                     State<M>& s) {
+    Gaps g;
+    step<M, FORCE>(C, c, gh, g1, s, g);
 }
 
 __device__ __forceinline__ void misfit_add(float U, float u, float& S, float& cS) {

@@ -13,25 +13,22 @@
 #include "afm_device.cuh"
 #include "afm_launch.h"
 #include "afm_tangent.cuh"
+#include "afm_warp.cuh"
+#include "kern_lm.cuh"
 
 namespace afm {
 
 namespace {
 
 template <typename F>
-cudaError_t dispatch_mfd(int m, int force, int D, F&& f) {
-    auto byD = [&](auto Mc, auto Fc) -> cudaError_t {
-        if (D <= 2) return f(Mc, Fc, std::integral_constant<int, 2>{});
-        if (D <= 4) return f(Mc, Fc, std::integral_constant<int, 4>{});
-        return f(Mc, Fc, std::integral_constant<int, AFM_MAXD>{});
-    };
+cudaError_t dispatch_mf(int m, int force, F&& f) {
     auto byF = [&](auto Mc) -> cudaError_t {
         switch (force) {
-            case F_LINEAR: return byD(Mc, std::integral_constant<int, F_LINEAR>{});
-            case F_DMT: return byD(Mc, std::integral_constant<int, F_DMT>{});
-            case F_DMT_KV: return byD(Mc, std::integral_constant<int, F_DMT_KV>{});
-            case F_HOOKE: return byD(Mc, std::integral_constant<int, F_HOOKE>{});
-            case F_SPRING_DAMPER: return byD(Mc, std::integral_constant<int, F_SPRING_DAMPER>{});
+            case F_LINEAR: return f(Mc, std::integral_constant<int, F_LINEAR>{});
+            case F_DMT: return f(Mc, std::integral_constant<int, F_DMT>{});
+            case F_DMT_KV: return f(Mc, std::integral_constant<int, F_DMT_KV>{});
+            case F_HOOKE: return f(Mc, std::integral_constant<int, F_HOOKE>{});
+            case F_SPRING_DAMPER: return f(Mc, std::integral_constant<int, F_SPRING_DAMPER>{});
         }
         return cudaErrorInvalidValue;
     };
@@ -40,17 +37,23 @@ cudaError_t dispatch_mfd(int m, int force, int D, F&& f) {
     return byF(std::integral_constant<int, AFM_MAXM>{});
 }
 
-constexpr int kThreads = 32;
+constexpr int kThreads = 128;   // (32: the drive table, built by one warp, costs 10 % more)
 constexpr int kFold = 32;   // steps summed in FP32 before folding into FP64 totals
 
 }  // namespace
 
 // Sensitivity pass of one particle per thread: S (as the forward kernel),
-// H [P][D][D] and b [P][D] in FP64.  Ragged form as the adjoint: off !=
-// nullptr gives particle p the record of pixel order[p / per_slot].
+// H [P][D][D] and b [P][D] in FP64.  CS: the tangents run along the law's
+// coefficients (afm_tangent.cuh), else along ND free parameters.  Ragged
+// form as the adjoint: off != nullptr gives particle p the record of pixel
+// order[p / per_slot].
 // PP (ragged form only): each particle's pixel has its own constants and
 // drive table (pix), read from global memory.
-template <int M, int FORCE, int ND, bool PP>
+// FMA-pipe bound when wide: DMT with 3 modes issues ~380 FP32 operations per
+// step (147 the solve, ~30 the partials, 3 x 65 the tangents, 9 the sums;
+// ~640 with parameter directions and linearised stages).  16 384 candidates x
+// 1 280 steps: 432 us, 696 us so.
+template <int M, int FORCE, int ND, bool CS, bool PP>
 __global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
                                                         const float* __restrict__ x, int P,
                                                         const float* __restrict__ U,
@@ -60,8 +63,10 @@ __global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
                                                         double* __restrict__ H_out,
                                                         double* __restrict__ b_out,
                                                         const PixConst pixc) {
+    constexpr int NH = ND * (ND + 1) / 2, NC = aff::CoefDirs<FORCE>::n;
+    static_assert(!CS || ND == NC, "coefficient directions");
     extern __shared__ __align__(16) float tabs[];
-    __shared__ double accH[ND * (ND + 1) / 2][kThreads], accb[ND][kThreads];
+    __shared__ double accH[NH][kThreads], accb[ND][kThreads];
     if constexpr (!PP) {
         build_drive_table(K0, tabs);
         __syncthreads();
@@ -87,61 +92,78 @@ __global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
     float xd[AFM_MAXD];
     for (int d = 0; d < AFM_MAXD; ++d) xd[d] = d < D ? x[(size_t)d * P + p] : 0.f;
     const Coef<float> c = make_coef<float, float>(K, xd);
-    float Jc[4][ND];
-    {
+    float Jc[NC][CS ? 1 : ND];
+    if constexpr (!CS) {
         double Jd[4][AFM_MAXD];
         coef_jacobian<float>(K, xd, Jd);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < NC; ++k)
 #pragma unroll
-            for (int e = 0; e < ND; ++e) Jc[k][e] = e < D ? (float)Jd[k][e] : 0.f;
+            for (int e = 0; e < ND; ++e)
+                Jc[k][e] = e < D ? (float)Jd[aff::CoefDirs<FORCE>::index(k)][e] : 0.f;
     }
-    float q[M], v[M], cq[M], cv[M], tq[ND][M], tv[ND][M];
-    init_state<float, M>(K, q, v, cq, cv);
+    const warp::Modes<M> C = warp::modes<M>(K);
+    warp::State<M> st;
+    warp::init<M>(K, C, tab[0], st);
+    aff::Tangent<M> tg[ND];
 #pragma unroll
-    for (int e = 0; e < ND; ++e)
+    for (int e = 0; e < ND; ++e) aff::zero(tg[e]);
 #pragma unroll
-        for (int i = 0; i < M; ++i) tq[e][i] = tv[e][i] = 0.f;
-#pragma unroll
-    for (int t = 0; t < ND * (ND + 1) / 2; ++t) accH[t][tid] = 0.0;
+    for (int t = 0; t < NH; ++t) accH[t][tid] = 0.0;
 #pragma unroll
     for (int e = 0; e < ND; ++e) accb[e][tid] = 0.0;
-    float hc[ND * (ND + 1) / 2], bc[ND];
+    float hc[NH], bc[ND];
 #pragma unroll
-    for (int t = 0; t < ND * (ND + 1) / 2; ++t) hc[t] = 0.f;
+    for (int t = 0; t < NH; ++t) hc[t] = 0.f;
 #pragma unroll
     for (int e = 0; e < ND; ++e) bc[e] = 0.f;
     float S = 0.f, cS = 0.f;
     int j = 0, fold = 0;
     const int spc2 = K.spc2;
+    float Un = n > 0 ? U[0] : 0.f;
     for (int s = 0; s < n; ++s) {
-        const float g0 = tab[j], gh = tab[j + 1], g1 = tab[j + 2];
+        const float gh = tab[j + 1], g1 = tab[j + 2];
         j += 2;
         if (j >= spc2) j = 0;
-        rk4_step_tl<M, FORCE, ND>(K, c, Jc, q, v, cq, cv, tq, tv, g0, gh, g1);
-        const float u = tip_sum<float, M>(q);
-        const float r = U[s] - u;
-        const float y = fmaf(r, r, -cS);
-        const float t = add_rn(S, y);
-        cS = sub_rn(sub_rn(t, S), y);
-        S = t;
-        float au[ND];
+        const float Unext = s + 1 < n ? U[s + 1] : 0.f;
+        warp::Gaps g;
+        warp::step<M, FORCE>(C, c, gh, g1, st, g);
+        aff::Partials<FORCE> Ps[4];
 #pragma unroll
-        for (int e = 0; e < ND; ++e) au[e] = tip_sum<float, M>(tq[e]);
+        for (int k = 0; k < 4; ++k) aff::partials<FORCE>(c, g.d[k], g.r[k], Ps[k]);
+        const float r = __fsub_rn(Un, st.u);
+        warp::misfit_add(Un, st.u, S, cS);
+        Un = Unext;
+#pragma unroll
+        for (int e = 0; e < ND; ++e) {
+            float G[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if constexpr (CS) {
+                    G[k] = Ps[k].Fc[e];
+                } else {
+                    G[k] = aff::mul(Ps[k].Fc[0], Jc[0][e]);
+#pragma unroll
+                    for (int l = 1; l < NC; ++l) G[k] = aff::fma(Ps[k].Fc[l], Jc[l][e], G[k]);
+                }
+            }
+            aff::tangent_step<M, FORCE>(K, Ps, G, tg[e]);
+        }
         int w = 0;
 #pragma unroll
         for (int e = 0; e < ND; ++e) {
-            bc[e] = fmaf(au[e], r, bc[e]);
+            const float ae = aff::tip(tg[e]);
+            bc[e] = aff::fma(ae, r, bc[e]);
 #pragma unroll
             for (int f = 0; f <= e; ++f) {
-                hc[w] = fmaf(au[e], au[f], hc[w]);
+                hc[w] = aff::fma(ae, aff::tip(tg[f]), hc[w]);
                 ++w;
             }
         }
         if (++fold == kFold || s + 1 == n) {
             fold = 0;
 #pragma unroll
-            for (int t2 = 0; t2 < ND * (ND + 1) / 2; ++t2) {
+            for (int t2 = 0; t2 < NH; ++t2) {
                 accH[t2][tid] += (double)hc[t2];
                 hc[t2] = 0.f;
             }
@@ -155,16 +177,27 @@ __global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
     if (!(S < INFINITY)) S = INFINITY;
     S_out[p] = S;
     double* H = H_out + (size_t)p * D * D;
-    int w = 0;
-    for (int e = 0; e < ND; ++e) {
-        for (int f = 0; f <= e; ++f) {
-            if (e < D) {
-                H[e * D + f] = accH[w][tid];
-                H[f * D + e] = accH[w][tid];
+    double* b = b_out + (size_t)p * D;
+    if constexpr (CS) {
+        double Hc[NH], bd[ND], Jd[4][AFM_MAXD];
+        coef_jacobian<float>(K, xd, Jd);
+#pragma unroll
+        for (int t = 0; t < NH; ++t) Hc[t] = accH[t][tid];
+#pragma unroll
+        for (int e = 0; e < ND; ++e) bd[e] = accb[e][tid];
+        for (int e = 0; e < D; ++e) aff::map_row<FORCE>(Jd, Hc, bd, D, e, H, b);
+    } else {
+        int w = 0;
+        for (int e = 0; e < ND; ++e) {
+            for (int f = 0; f <= e; ++f) {
+                if (e < D) {
+                    H[e * D + f] = accH[w][tid];
+                    H[f * D + e] = accH[w][tid];
+                }
+                ++w;
             }
-            ++w;
+            if (e < D) b[e] = accb[e][tid];
         }
-        if (e < D) b_out[(size_t)p * D + e] = accb[e][tid];
     }
 }
 
@@ -272,15 +305,14 @@ cudaError_t launch_sens(const KConst<float>& K, const float* x, int P, const flo
                         int per_slot, const PixConst& pix) {
     const bool pp = pix.kf != nullptr;
     if (pp && off == nullptr) return cudaErrorInvalidValue;
-    if (!pp && sens_modes_supported(K.m, K.force, P, K.D))
-        return launch_sens_modes(K, x, P, U, S, H, b, st, off, order, per_slot);
     if (!pp && sens_lanes_preferred(P, K.D))
         return launch_sens_lanes(K, x, P, U, S, H, b, st, off, order, per_slot);
     const int blocks = (P + kThreads - 1) / kThreads;
-    const size_t smem = pp ? 0 : sizeof(float) * (size_t)(K.spc2 + 1);
-    return dispatch_mfd(K.m, K.force, K.D, [&](auto Mc, auto Fc, auto Dc) -> cudaError_t {
-        auto go = [&](auto Pc) -> cudaError_t {
-            auto kern = sens_kernel<decltype(Mc)::value, decltype(Fc)::value, decltype(Dc)::value,
+    return dispatch_mf(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
+        constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;
+        const size_t smem = pp ? 0 : sizeof(float) * (size_t)(K.spc2 + 1);
+        auto go = [&](auto Dc, auto Cc, auto Pc) -> cudaError_t {
+            auto kern = sens_kernel<M, FORCE, decltype(Dc)::value, decltype(Cc)::value,
                                     decltype(Pc)::value>;
             if (smem > 24 * 1024) {
                 cudaError_t e = cudaFuncSetAttribute(
@@ -290,7 +322,9 @@ cudaError_t launch_sens(const KConst<float>& K, const float* x, int P, const flo
             kern<<<blocks, kThreads, smem, st>>>(K, x, P, U, off, order, per_slot, S, H, b, pix);
             return cudaGetLastError();
         };
-        return pp ? go(std::true_type{}) : go(std::false_type{});
+        return sens_dirs<FORCE>(K.D, [&](auto Dc, auto Cc) -> cudaError_t {
+            return pp ? go(Dc, Cc, std::true_type{}) : go(Dc, Cc, std::false_type{});
+        });
     });
 }
 
