@@ -421,6 +421,38 @@ bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
 // Sturm bisection of L^-1 K L^-T), Rayleigh damping, the free steady state
 // (complex solve) as initial state, and the drive table scale.
 // ---------------------------------------------------------------------------
+// All of the set-up is on the host path of every FE call, so its cost matters
+// beside a 5 ms launch: 14 ms for 64 DOFs when every loop ran over full
+// matrices one row and one eigenvalue at a time, most of it products of the
+// compensated Rayleigh quotients with the zeros of the banded M and K.
+// Products with exact zeros are skipped and independent sums and bisections
+// run side by side; every sum keeps its terms and their order.
+constexpr int kBand = 3;   // element matrices couple DOFs at most 3 apart
+
+// out[i] = sum_j A[i][j] v[j], four rows' sums side by side.
+void row_products(const double* A, const double* v, int n, double* out) {
+    int i = 0;
+    for (; i + 4 <= n; i += 4) {
+        const double *a = A + (size_t)i * n, *b = a + n, *c = b + n, *d = c + n;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        for (int j = 0; j < n; ++j) {
+            s0 += a[j] * v[j];
+            s1 += b[j] * v[j];
+            s2 += c[j] * v[j];
+            s3 += d[j] * v[j];
+        }
+        out[i] = s0;
+        out[i + 1] = s1;
+        out[i + 2] = s2;
+        out[i + 3] = s3;
+    }
+    for (; i < n; ++i) {
+        double t = 0.0;
+        for (int j = 0; j < n; ++j) t += A[(size_t)i * n + j] * v[j];
+        out[i] = t;
+    }
+}
+
 // Householder reduction of the symmetric A (row-major, destroyed) to
 // tridiagonal (d, e), accumulating the orthogonal Q with A_orig = Q T Q^T.
 void householder_tridiag(std::vector<double>& A, int n, std::vector<double>& d,
@@ -439,11 +471,8 @@ void householder_tridiag(std::vector<double>& A, int n, std::vector<double>& d,
         double vn2 = 0.0;
         for (int i = 0; i < n; ++i) vn2 += v[i] * v[i];
         if (vn2 == 0.0) continue;
-        for (int i = 0; i < n; ++i) {
-            double t = 0.0;
-            for (int j = 0; j < n; ++j) t += A[(size_t)i * n + j] * v[j];
-            p[i] = 2.0 * t / vn2;
-        }
+        row_products(A.data(), v.data(), n, p.data());
+        for (int i = 0; i < n; ++i) p[i] = 2.0 * p[i] / vn2;
         double K = 0.0;
         for (int i = 0; i < n; ++i) K += v[i] * p[i];
         K /= vn2;
@@ -451,10 +480,9 @@ void householder_tridiag(std::vector<double>& A, int n, std::vector<double>& d,
         for (int i = 0; i < n; ++i)
             for (int j = 0; j < n; ++j) A[(size_t)i * n + j] -= v[i] * q[j] + q[i] * v[j];
         // Q <- Q H, H = I - 2 v v^T / |v|^2
+        row_products(Q.data(), v.data(), n, q.data());
         for (int i = 0; i < n; ++i) {
-            double t = 0.0;
-            for (int j = 0; j < n; ++j) t += Q[(size_t)i * n + j] * v[j];
-            t *= 2.0 / vn2;
+            const double t = q[i] * (2.0 / vn2);
             for (int j = 0; j < n; ++j) Q[(size_t)i * n + j] -= t * v[j];
         }
     }
@@ -464,33 +492,54 @@ void householder_tridiag(std::vector<double>& A, int n, std::vector<double>& d,
     for (int i = 0; i + 1 < n; ++i) e[i] = A[(size_t)(i + 1) * n + i];
 }
 
-int sturm_count(const std::vector<double>& d, const std::vector<double>& e, double x) {
-    int cnt = 0;
-    double q = d[0] - x;
-    if (q < 0) ++cnt;
-    for (size_t i = 1; i < d.size(); ++i) {
-        if (q == 0.0) q = 1e-300;
-        q = d[i] - x - e[i - 1] * e[i - 1] / q;
-        if (q < 0) ++cnt;
-    }
-    return cnt;
-}
-
-// k-th smallest eigenvalue of the tridiagonal (d, e) by Sturm bisection.
-double kth_eigenvalue(const std::vector<double>& d, const std::vector<double>& e, int k) {
-    double lo = 1e300, hi = -1e300;
+// The eigenvalues of the tridiagonal (d, e) in ascending order, by Sturm
+// bisection: kLanes bisections side by side, so that their divisions overlap.
+void eigenvalues(const std::vector<double>& d, const std::vector<double>& e,
+                 std::vector<double>& lam) {
+    constexpr int kLanes = 16;
     const int n = (int)d.size();
+    double lo0 = 1e300, hi0 = -1e300;
     for (int i = 0; i < n; ++i) {
         double r = (i > 0 ? std::fabs(e[i - 1]) : 0.0) + (i + 1 < n ? std::fabs(e[i]) : 0.0);
-        lo = std::min(lo, d[i] - r);
-        hi = std::max(hi, d[i] + r);
+        lo0 = std::min(lo0, d[i] - r);
+        hi0 = std::max(hi0, d[i] + r);
     }
-    for (int it = 0; it < 400; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        if (sturm_count(d, e, mid) > k) hi = mid; else lo = mid;
-        if (hi - lo <= 1e-16 * std::fabs(hi)) break;
+    lam.assign(n, 0.0);
+    for (int k0 = 0; k0 < n; k0 += kLanes) {
+        const int m = std::min(kLanes, n - k0);
+        double lo[kLanes], hi[kLanes], mid[kLanes], q[kLanes];
+        int cnt[kLanes];
+        bool done[kLanes] = {};
+        for (int k = 0; k < kLanes; ++k) {
+            lo[k] = lo0;
+            hi[k] = hi0;
+        }
+        int left = m;
+        for (int it = 0; it < 400 && left > 0; ++it) {
+            for (int k = 0; k < kLanes; ++k) {
+                mid[k] = 0.5 * (lo[k] + hi[k]);
+                q[k] = d[0] - mid[k];
+                cnt[k] = q[k] < 0 ? 1 : 0;
+            }
+            for (int i = 1; i < n; ++i) {
+                const double di = d[i], ee = e[i - 1];
+                for (int k = 0; k < kLanes; ++k) {
+                    const double qk = q[k] == 0.0 ? 1e-300 : q[k];
+                    q[k] = di - mid[k] - ee * ee / qk;
+                    cnt[k] += q[k] < 0 ? 1 : 0;
+                }
+            }
+            for (int k = 0; k < m; ++k) {
+                if (done[k]) continue;
+                if (cnt[k] > k0 + k) hi[k] = mid[k]; else lo[k] = mid[k];
+                if (hi[k] - lo[k] <= 1e-16 * std::fabs(hi[k])) {
+                    done[k] = true;
+                    --left;
+                }
+            }
+        }
+        for (int k = 0; k < m; ++k) lam[k0 + k] = 0.5 * (lo[k] + hi[k]);
     }
-    return 0.5 * (lo + hi);
 }
 
 // Eigenvector of the tridiagonal (d, e) for eigenvalue lam, by two steps of
@@ -557,7 +606,7 @@ struct CompSum {
 };
 
 // Rayleigh quotient phi^T K phi / phi^T M phi of an eigenvector, both forms
-// accumulated with compensation.  The lowest eigenvalues of a stiff FE pair
+// accumulated with compensation over the band.  The lowest eigenvalues of a stiff FE pair
 // come out of an FP64 eigensolver with relative errors ~ eps * lambda_max /
 // lambda (a few 1e-9 for 32 elements); the quotient of the computed vector
 // is exact to rounding (its error is quadratic in the vector's), which keeps
@@ -567,7 +616,7 @@ double rayleigh_quotient(const std::vector<double>& K, const std::vector<double>
     CompSum num, den;
     for (int i = 0; i < n; ++i) {
         CompSum kp, mp;
-        for (int j = 0; j < n; ++j) {
+        for (int j = std::max(0, i - kBand); j <= std::min(n - 1, i + kBand); ++j) {
             const double pj = Phi[(size_t)j * n + md];
             kp.add_prod(K[(size_t)i * n + j], pj);
             mp.add_prod(M[(size_t)i * n + j], pj);
@@ -610,7 +659,8 @@ afm_status fe_setup(const afm_problem& pr, int spc, int n_steps, afm::FeConst& F
     for (int i = 0; i < n; ++i)
         for (int j = 0; j <= i; ++j) {
             double s2 = M[(size_t)i * n + j];
-            for (int q = 0; q < j; ++q) s2 -= Lc[(size_t)i * n + q] * Lc[(size_t)j * n + q];
+            for (int q = std::max(0, i - kBand); q < j; ++q)
+                s2 -= Lc[(size_t)i * n + q] * Lc[(size_t)j * n + q];
             if (i == j) {
                 if (!(s2 > 0)) return fail(AFM_ERR_INVALID_ARG, "FE mass matrix not positive definite");
                 Lc[(size_t)i * n + i] = std::sqrt(s2);
@@ -622,30 +672,28 @@ afm_status fe_setup(const afm_problem& pr, int spc, int n_steps, afm::FeConst& F
     for (int col = 0; col < n; ++col)
         for (int i = 0; i < n; ++i) {
             double s2 = K[(size_t)i * n + col];
-            for (int q = 0; q < i; ++q) s2 -= Lc[(size_t)i * n + q] * T[(size_t)q * n + col];
+            for (int q = std::max(0, i - kBand); q < i; ++q)
+                s2 -= Lc[(size_t)i * n + q] * T[(size_t)q * n + col];
             T[(size_t)i * n + col] = s2 / Lc[(size_t)i * n + i];
         }
     for (int row = 0; row < n; ++row)
         for (int i = 0; i < n; ++i) {
             double s2 = T[(size_t)row * n + i];
-            for (int q = 0; q < i; ++q) s2 -= Lc[(size_t)i * n + q] * B[(size_t)row * n + q];
+            for (int q = std::max(0, i - kBand); q < i; ++q)
+                s2 -= Lc[(size_t)i * n + q] * B[(size_t)row * n + q];
             B[(size_t)row * n + i] = s2 / Lc[(size_t)i * n + i];
         }
     std::vector<double> d, e, Q;
     householder_tridiag(B, n, d, e, Q);
-    std::vector<double> lam(n), Phi((size_t)n * n);   // Phi[i * n + mode]
+    std::vector<double> lam, Phi((size_t)n * n);   // Phi[i * n + mode]
     std::vector<double> y, wv(n);
+    eigenvalues(d, e, lam);
     for (int md = 0; md < n; ++md) {
-        lam[md] = kth_eigenvalue(d, e, md);
         tridiag_eigvec(d, e, lam[md], y);
-        for (int i = 0; i < n; ++i) {
-            double t = 0.0;
-            for (int j = 0; j < n; ++j) t += Q[(size_t)i * n + j] * y[j];
-            wv[i] = t;
-        }
+        row_products(Q.data(), y.data(), n, wv.data());
         for (int i = n - 1; i >= 0; --i) {   // Lc^T phi = w
             double t = wv[i];
-            for (int j = i + 1; j < n; ++j) t -= Lc[(size_t)j * n + i] * Phi[(size_t)j * n + md];
+            for (int j = i + 1; j <= std::min(n - 1, i + kBand); ++j) t -= Lc[(size_t)j * n + i] * Phi[(size_t)j * n + md];
             Phi[(size_t)i * n + md] = t / Lc[(size_t)i * n + i];
         }
         lam[md] = rayleigh_quotient(K, M, n, Phi, md);
