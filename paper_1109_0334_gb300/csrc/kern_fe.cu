@@ -12,10 +12,13 @@
 // a condition number of ~3e4, which turns FP32 (and TF32) rounding into
 // 1e-3 errors of the resonant response.
 //
-// Layout: AFM_FE_LANES lanes per particle, each lane owns modes
-// lane, lane + 8, ... and holds their step coefficients in registers; the
-// tip deflection is a group sum (3 shuffles), the Newton solve for the tip
-// force runs redundantly in the group's lanes.
+// Layout: 4 or 8 lanes per particle, each lane owns modes lane, lane + lanes,
+// ... and holds their step coefficients in registers; the tip deflection is a
+// group sum (2 or 3 shuffles), the Newton solve for the tip force runs
+// redundantly in the group's lanes.  Per mode and step 8 FP32 operations (the
+// compensated ones 17): bound by instruction issue with four warps on a
+// sub-partition, by the chain of one step (sum, shuffles, two force
+// evaluations) with fewer.
 //
 // The kernel carries each mode scaled by its tip displacement, w_i =
 // phi_i(tip) z_i.  The recursion is linear and homogeneous in (z_i, delta_i),
@@ -35,24 +38,27 @@ constexpr int FEN = AFM_FE_MAXN;
 // left 48 SMs with half the load of the others)
 constexpr int FE_THREADS = 64;
 constexpr int FE_MIN_BLOCKS = 8;   // caps registers at 128 per thread
-// lanes per particle: AFM_FE_LANES in FP32 (throughput), a whole warp in FP64
-// (latency: one trajectory, the FP64 re-evaluation)
-template <typename T>
-struct FeLanes {
-    static constexpr int value = sizeof(T) == 8 ? 32 : AFM_FE_LANES;
-};
+constexpr int FE_MIN_BLOCKS4 = 4;  // 4 lanes: 16 modes per lane take 167 registers
+// Lanes per particle of the FP64 kernels: a whole warp (latency: one
+// trajectory, the FP64 re-evaluation).  FP32: 4 or 8, see fe_lanes32.
+constexpr int FE_LANES64 = 32;
 
-// Which mode slots of a lane take compensated updates.  FP64: all.  FP32:
-// slot 0 only, the lowest AFM_FE_LANES modes, which hold the resonant
+// Which mode slots of a lane take compensated updates.  FP64: all.  FP32: the
+// lowest AFM_FE_LANES modes, which hold the resonant
 // response and whose step increment is a small fraction of the coordinate
 // (omega h << 1), so that plain sums lose its low bits every step.  The
 // stiff modes above respond quasi-statically with amplitudes ~(omega_1 /
 // omega_i)^2 of the first mode's forced term and omega h ~ 1: their rounding
 // stays far below FP32 resolution of the tip deflection.
-template <typename T>
+template <typename T, int FEL>
 __host__ __device__ constexpr bool fe_comp(int j) {
-    return sizeof(T) == 8 || j == 0;
+    return sizeof(T) == 8 || j * FEL < AFM_FE_LANES;
 }
+
+// Keeps a coefficient in its register: the compiler may otherwise form it
+// again from its FP64 factors in every step.
+__device__ __forceinline__ void pin(float& v) { asm volatile("" : "+f"(v)); }
+__device__ __forceinline__ void pin(double& v) { asm volatile("" : "+d"(v)); }
 
 // Drive term of the Newmark step at phase index j of the period: the base
 // acceleration enters as y(t+) + 2 y(t) + y(t-), evaluated in FP64.
@@ -75,6 +81,21 @@ __device__ __forceinline__ void fe_force(const Coef<T>& c, T d, T& Fv, T& dF) {
     if (FORCE == F_LINEAR) {
         Fv = -c.c0 * (d - c.c1);
         dF = -c.c0;
+    } else if (FORCE == F_DMT && sizeof(T) == 8) {
+        // a reciprocal out of contact or a square root in it, not both (352 and
+        // 618 clocks); the trajectory's warp takes one branch
+        if (d > c.c3) {
+            const T r = rcp_fast(d);
+            const T r2 = r * r;
+            Fv = -(c.c1 * r2);
+            dF = (T)2 * c.c1 * r2 * r;
+        } else {
+            const T r = rcp_fast(c.c3);
+            const T r2 = r * r;
+            const T del = fmax(c.c3 - d, (T)0), sq = sqrt_fast(del);
+            Fv = c.c0 * del * sq - c.c1 * r2;
+            dF = (T)(-1.5) * c.c0 * sq;
+        }
     } else if (FORCE == F_DMT) {
         // branch-free (the van der Waals term saturates at d = a0, where it
         // is the contact branch's constant): particles of one warp in and out
@@ -130,12 +151,11 @@ __device__ __forceinline__ T fe_newton(const Coef<T>& c, T Zc, T base, T cz, T F
 // iteration (PSO move, forward, personal/global best; T = float);
 // MODE 2: FP64 re-evaluation of an inversion's winner into afm_result.
 // ---------------------------------------------------------------------------
-template <typename T, typename TU, int FORCE, int MODE>
-__global__ void __launch_bounds__(FE_THREADS, FE_MIN_BLOCKS) fe_modal_kernel(
+template <typename T, typename TU, int FORCE, int MODE, int FEL>
+__global__ void __launch_bounds__(FE_THREADS, FEL == 4 ? FE_MIN_BLOCKS4 : FE_MIN_BLOCKS) fe_modal_kernel(
     const FeConst F, const PsoConst pc, SwarmPtrs sw, const T* __restrict__ xin, int P,
     T* __restrict__ defl, const TU* __restrict__ U, T* __restrict__ S_out,
     float* __restrict__ history, int it, afm_result* __restrict__ res) {
-    constexpr int FEL = FeLanes<T>::value;
     constexpr int FEM = FEN / FEL;               // modes per lane
     constexpr int FE_PPB = FE_THREADS / FEL;     // particles per block
     extern __shared__ __align__(16) unsigned char fe_smem[];
@@ -200,25 +220,32 @@ __global__ void __launch_bounds__(FE_THREADS, FE_MIN_BLOCKS) fe_modal_kernel(
     __syncthreads();
 
     // ---- this lane's modes: coefficients and tip-scaled state
+    constexpr int NC = sizeof(T) == 8 ? FEM : AFM_FE_LANES / FEL;   // compensated slots (the first)
     T b1[FEM], d2[FEM], gq[FEM], fq[FEM];
-    T z[FEM], dz[FEM], cz[FEM], cdz[FEM];
+    T z[FEM], dz[FEM], cz[NC], cdz[NC], b1lo[NC];
 #pragma unroll
     for (int j = 0; j < FEM; ++j) {
         const int i = lane + FEL * j;
         const double pt = F.pt[i];
         b1[j] = (T)F.b1[i];
         // the uncompensated slots take 1 + d2, see the step below
-        d2[j] = fe_comp<T>(j) ? (T)F.d2[i] : (T)(1.0 + F.d2[i]);
+        d2[j] = fe_comp<T, FEL>(j) ? (T)F.d2[i] : (T)(1.0 + F.d2[i]);
         gq[j] = (T)(F.g[i] * pt);
         fq[j] = (T)(F.f[i] * pt);
+        pin(b1[j]);
+        pin(d2[j]);
+        pin(gq[j]);
+        pin(fq[j]);
         z[j] = (T)(F.z0[i] * pt);
         dz[j] = (T)(F.dz0[i] * pt);
-        cz[j] = (T)0;
-        cdz[j] = (T)0;
+        if (j < NC) {
+            cz[j < NC ? j : 0] = (T)0;
+            cdz[j < NC ? j : 0] = (T)0;
+            // the low word of the lowest modes' b1 (the resonant frequency must
+            // be represented to ~1e-12); zero in FP64
+            b1lo[j < NC ? j : 0] = (T)(F.b1[i] - (double)b1[j]);
+        }
     }
-    // the low word of the lowest mode's b1 (the resonant frequency must be
-    // represented to ~1e-12); zero in FP64
-    const T b1lo = (T)(F.b1[lane] - (double)b1[0]);
     const T Zc = (T)F.Zc, ctip = (T)F.ctip;
     T Fn, Fm, dF;
     fe_force<FORCE, T>(cfc, Zc + (T)F.utip0, Fn, dF);
@@ -246,15 +273,19 @@ __global__ void __launch_bounds__(FE_THREADS, FE_MIN_BLOCKS) fe_modal_kernel(
         // the drive and past-force terms first: they wait on no state update
         // of the previous step.  Compensated slots form the increment; the
         // others form delta_n + increment in one sum, with (1 + d2) dz.
+        // (Taking the others' force terms together after the Newton solve
+        // saves one operation of 8 per mode, but adds them to the large end of
+        // the sum: the misfits' error against FP64 grew 1.5 times.)
         T incs[FEM], zps[FEM];
 #pragma unroll
         for (int j = 0; j < FEM; ++j) {
+            const int k = j < NC ? j : 0;
             T inc = fma(fq[j], Fo, gq[j] * G);
             inc = fma(d2[j], dz[j], inc);
-            if (j == 0) inc = fma(b1lo, z[j], inc);
+            if (sizeof(T) == 8 ? j == 0 : fe_comp<T, FEL>(j)) inc = fma(b1lo[k], z[j], inc);
             inc = fma(b1[j], z[j], inc);
             incs[j] = inc;
-            zps[j] = fe_comp<T>(j) ? z[j] + ((dz[j] + inc) - cz[j]) : z[j] + inc;
+            zps[j] = fe_comp<T, FEL>(j) ? z[j] + ((dz[j] + inc) - cz[k]) : z[j] + inc;
         }
         T tsum = fe_sum<T, FEM>(zps);
 #pragma unroll
@@ -265,9 +296,10 @@ __global__ void __launch_bounds__(FE_THREADS, FE_MIN_BLOCKS) fe_modal_kernel(
         // (in FP32 for the lowest modes only)
 #pragma unroll
         for (int j = 0; j < FEM; ++j) {
-            if (fe_comp<T>(j)) {
-                kahan_add(dz[j], cdz[j], fma(fq[j], Fp, incs[j]));
-                kahan_add(z[j], cz[j], dz[j]);
+            if (fe_comp<T, FEL>(j)) {
+                const int k = j < NC ? j : 0;
+                kahan_add(dz[j], cdz[k], fma(fq[j], Fp, incs[j]));
+                kahan_add(z[j], cz[k], dz[j]);
             } else {
                 dz[j] = fma(fq[j], Fp, incs[j]);
                 z[j] = z[j] + dz[j];
@@ -364,12 +396,12 @@ size_t fe_smem(const FeConst& F) {
     return sizeof(T) * (size_t)F.spc;
 }
 
-template <typename T, typename TU, int MODE, typename... Args>
+template <typename T, typename TU, int MODE, int FEL, typename... Args>
 cudaError_t fe_launch(const FeConst& F, int blocks, cudaStream_t st, Args... args) {
     const int threads = MODE == 2 ? 32 : FE_THREADS;   // the FP64 re-evaluation: one warp
     const size_t smem = fe_smem<T>(F);
     return fe_dispatch(F.pm.force, [&](auto Fc) -> cudaError_t {
-        auto kern = fe_modal_kernel<T, TU, decltype(Fc)::value, MODE>;
+        auto kern = fe_modal_kernel<T, TU, decltype(Fc)::value, MODE, FEL>;
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
@@ -379,39 +411,61 @@ cudaError_t fe_launch(const FeConst& F, int blocks, cudaStream_t st, Args... arg
     });
 }
 
+int fe_blocks(int P, int lanes) {
+    const int ppb = FE_THREADS / lanes;
+    return (P + ppb - 1) / ppb;
+}
+
+// Lanes per particle in FP32.  8 lanes have the shorter step, 4 lanes half the
+// warps, and one Newton solve and tip sum for every 16 modes instead of 8.
+// Per step, 8 : 4 lanes, by warps of 8 lanes per sub-partition: up to 1 247 :
+// 277 ns, up to 2 304 : 277, up to 3 362 : 371, up to 4 436 : 376 (8 192
+// particles), 7 764 : 742 (16 384), 27 2 575 : 2 310 (65 536).
+int fe_lanes32(int P) {
+    const int w = (P + 2431) / 2432;   // 2432 particles x 8 lanes: a warp per sub-partition
+    return w == 2 || w >= 4 ? 4 : 8;
+}
+
 }  // namespace
 
 cudaError_t launch_fe_forward_f32(const FeConst& F, const float* x, int P, float* defl,
                                   const float* U, float* S, cudaStream_t st) {
     PsoConst pc{};
     SwarmPtrs sw{};
-    constexpr int ppb = FE_THREADS / FeLanes<float>::value;
-    return fe_launch<float, float, 0>(F, (P + ppb - 1) / ppb, st, pc, sw, x, P, defl, U, S,
-                                      (float*)nullptr, 0, (afm_result*)nullptr);
+    const int L = fe_lanes32(P);
+    auto go = [&](auto Lc) {
+        return fe_launch<float, float, 0, decltype(Lc)::value>(F, fe_blocks(P, L), st, pc, sw, x, P,
+                                                               defl, U, S, (float*)nullptr, 0,
+                                                               (afm_result*)nullptr);
+    };
+    return L == 4 ? go(std::integral_constant<int, 4>{}) : go(std::integral_constant<int, 8>{});
 }
 
 cudaError_t launch_fe_forward_f64(const FeConst& F, const double* x, int P, double* defl,
                                   const double* U, double* S, cudaStream_t st) {
     PsoConst pc{};
     SwarmPtrs sw{};
-    constexpr int ppb = FE_THREADS / FeLanes<double>::value;
-    return fe_launch<double, double, 0>(F, (P + ppb - 1) / ppb, st, pc, sw, x, P, defl, U,
-                                        S, (float*)nullptr, 0, (afm_result*)nullptr);
+    return fe_launch<double, double, 0, FE_LANES64>(F, fe_blocks(P, FE_LANES64), st, pc, sw, x, P,
+                                                    defl, U, S, (float*)nullptr, 0,
+                                                    (afm_result*)nullptr);
 }
 
 cudaError_t launch_fe_invert_iter(const FeConst& F, const PsoConst& pc, const SwarmPtrs& sw,
                                   const float* U, float* history, int it, cudaStream_t st) {
-    constexpr int ppb = FE_THREADS / FeLanes<float>::value;
-    return fe_launch<float, float, 1>(F, (pc.P + ppb - 1) / ppb, st, pc, sw,
-                                      (const float*)nullptr, pc.P, (float*)nullptr, U,
-                                      (float*)nullptr, history, it, (afm_result*)nullptr);
+    const int L = fe_lanes32(pc.P);
+    auto go = [&](auto Lc) {
+        return fe_launch<float, float, 1, decltype(Lc)::value>(
+            F, fe_blocks(pc.P, L), st, pc, sw, (const float*)nullptr, pc.P, (float*)nullptr, U,
+            (float*)nullptr, history, it, (afm_result*)nullptr);
+    };
+    return L == 4 ? go(std::integral_constant<int, 4>{}) : go(std::integral_constant<int, 8>{});
 }
 
 cudaError_t launch_fe_invert_final(const FeConst& F, const PsoConst& pc, const SwarmPtrs& sw,
                                    const float* U, float* history, void* result, cudaStream_t st) {
-    return fe_launch<double, float, 2>(F, 1, st, pc, sw, (const double*)nullptr, pc.P,
-                                       (double*)nullptr, U, (double*)nullptr, history, 0,
-                                       reinterpret_cast<afm_result*>(result));
+    return fe_launch<double, float, 2, FE_LANES64>(F, 1, st, pc, sw, (const double*)nullptr, pc.P,
+                                                   (double*)nullptr, U, (double*)nullptr, history,
+                                                   0, reinterpret_cast<afm_result*>(result));
 }
 
 }  // namespace afm
