@@ -7,7 +7,8 @@
 // through one fma each, so a step is two force evaluations deep.
 //
 // Used by the FP64 solves (kern_forward64.cu, the passes of afm_reeval.cuh),
-// the tangents (afm_tangent.cuh) and the FP32 guesses of the re-evaluation.
+// the tangents (afm_tangent.cuh), the adjoint of few particles
+// (kern_adjoint.cu) and the FP32 guesses of the re-evaluation.
 // The FP32 forward solves keep the stage form of afm_device.cuh: in FP32 the
 // two forms round differently, and a swarm's misfits would move by up to
 // 5e-5 of their value near the noise floor (the stage form's own distance
@@ -243,7 +244,11 @@ __device__ __forceinline__ void stages(const KConst<T>& K, const LawCoef<V>& c, 
                                        const State<V, M, COMP>& s, Stages<V>& g) {
     const Affine<T>& A = K.af;
     constexpr bool rate = UsesRate<FORCE>::value;
-    const V zq = add(K.Zc, s.q[0]);
+    // the gap is the small difference of Zc and q_0: in FP32 with every mode
+    // compensated (the adjoint) it takes q_0's lost bits, on which contact
+    // events and their slopes hang
+    V zq = add(K.Zc, s.q[0]);
+    if constexpr (COMP == ALL && sizeof(V) == 4) zq = sub(zq, s.cq[0]);
     g.d[0] = M > 1 ? add(zq, s.s1) : zq;
     V sp = (V)0, a;
     if constexpr (M > 1) {

@@ -1523,7 +1523,7 @@ afm_status afm_adjoint_workspace_size(const afm_problem* prob, int P, size_t* by
     afm_status st = check_problem(prob);
     if (st) return st;
     const int m = prob->model == AFM_POINT_MASS ? 1 : prob->n_modes;
-    *bytes = align256(sizeof(float) * afm::adjoint_ckpt_floats(m, prob->n_steps, P));
+    *bytes = align256(sizeof(float) * afm::adjoint_ws_floats(m, prob->force, prob->n_steps, P));
     return AFM_OK;
 }
 
@@ -1547,7 +1547,7 @@ afm_status afm_adjoint(afm_ctx* ctx, const afm_problem* prob, const float* x, in
     fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AFM_CUDA(timed_launch(ctx, s, [&] {
-                 return afm::launch_adjoint(K, x, P, U, S, dS_dx, static_cast<float*>(workspace), s);
+                 return afm::launch_adjoint_split(K, x, P, U, S, dS_dx, static_cast<float*>(workspace), s);
              }),
              "adjoint kernel");
     return AFM_OK;
