@@ -68,7 +68,9 @@ struct BatchArgs {
     const int* order;      // queue order of pixels (longest first) or nullptr
     int n_pix;
     uint32_t pixel0;       // Philox counter word 2 of pixel 0
-    int* queue;            // pixel counter (zeroed before the launch)
+    int* queue;            // batch_queue_words(n_pix) words, zeroed before the launch
+    int layer;             // > 0: a block per pixel on `layer` SMs, dealt by batch_deal;
+                           // 0: blocks pull pixels until the queue is empty
     afm_result* res;       // [n_pix]
     float* pb_out;         // nullptr, or per queue slot the final personal bests
                            // [D][P] (normalised cube) followed by their misfits [P]
@@ -81,6 +83,18 @@ struct BatchArgs {
     int n_seed;
     PixConst pix;          // per-pixel constants (pix.kf == nullptr: shared)
 };
+// Where every pixel has a resident block, slots (longest first) are dealt to
+// the SMs in layers of one slot per SM, to and fro, the last full layer
+// longest last: the SMs' sums are even or, where a rest follows, smaller on
+// the SMs that get one of it.  SM i's slot of layer l:
+__host__ __device__ inline int batch_deal(int l, int i, int n, int sms) {
+    const int full = n / sms;
+    return l * sms + (l < full && (full - l) % 2 ? sms - 1 - i : i);
+}
+// Words of BatchArgs::queue: counters, per SM (id modulo 256) its blocks and
+// its index, and for a dealt launch a flag per slot.
+constexpr int BATCH_SMS = 256, BATCH_FLAGS = 4 + 2 * BATCH_SMS;
+inline size_t batch_queue_words(int n_pix) { return (size_t)BATCH_FLAGS + (size_t)n_pix; }
 int batch_threads(int P, int kp);
 // largest block of the batch kernel with kp particles per thread (the
 // paired-instruction kernels of kp = 2, 4 are built for up to 128 registers)

@@ -952,7 +952,7 @@ BatchLayout batch_layout(int n_pix) {
     BatchLayout L;
     L.order = 0;
     L.queue = align256(sizeof(int) * (size_t)n_pix);
-    L.total = L.queue + 256;
+    L.total = L.queue + align256(sizeof(int) * afm::batch_queue_words(n_pix));
     return L;
 }
 
@@ -1064,8 +1064,9 @@ afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst
         probe.iters = 0;
         afm::BatchArgs pa = a;
         pa.n_pix = std::min(a.n_pix, ctx->num_sms * occ);
+        pa.layer = ctx->num_sms;
         const int grid = pa.n_pix;
-        AFM_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int), s), "cudaMemsetAsync");
+        AFM_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int) * afm::batch_queue_words(a.n_pix), s), "cudaMemsetAsync");
         AFM_CUDA(cudaEventRecord(e0, s), "cudaEventRecord");
         AFM_CUDA(afm::launch_batch(Kf, probe, pa, kp, grid, s), "batch probe kernel");
         AFM_CUDA(cudaEventRecord(e1, s), "cudaEventRecord");
@@ -1935,6 +1936,7 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
     }
     B.kp = kp;
     B.grid = std::min(a.n_pix, ctx->num_sms * occ);
+    a.layer = B.grid == a.n_pix ? ctx->num_sms : 0;
     if (particles_per_thread) *particles_per_thread = kp;
     return AFM_OK;
 }
@@ -1999,7 +2001,7 @@ afm_status afm_invert_batch(afm_ctx* ctx, const afm_problem* probs, int n_prob,
         cudaStream_t c = ctx->capture_stream;
         cudaError_t e = cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return drop(e, "begin capture");
-        e = cudaMemsetAsync(a.queue, 0, sizeof(int), c);
+        e = cudaMemsetAsync(a.queue, 0, sizeof(int) * afm::batch_queue_words(a.n_pix), c);
         if (e == cudaSuccess && a.order) e = afm::batch_sort(off, n_pix, const_cast<int*>(a.order), c);
         if (e == cudaSuccess) e = cudaEventRecordWithFlags(g.ev_own[0], c, cudaEventRecordExternal);
         if (e == cudaSuccess) e = afm::launch_batch(Kf, pc, a, kp, grid, c);
@@ -2159,7 +2161,7 @@ static afm_status batch_polished_run(afm_ctx* ctx, const afm_problem* prob, cons
     float* Sk = reinterpret_cast<float*>(ws + PL.Sk);
     int* ik = reinterpret_cast<int*>(ws + PL.ik);
     const int D = prob->n_free, Kc = polish_k, J = n_cand, Nt = n_pix * Kc;
-    AFM_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int), s), "cudaMemsetAsync");
+    AFM_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int) * afm::batch_queue_words(a.n_pix), s), "cudaMemsetAsync");
     AFM_CUDA(timed_launch(ctx, s, [&] { return afm::launch_batch(B.Kf, B.pc, a, B.kp, B.grid, s); }),
              "batch kernel");
     AFM_CUDA(afm::launch_topk_pix(a.pb_out, n_pix, cfg->P, D, Kc, xk, Sk, ik, s), "top-k kernel");

@@ -6,6 +6,7 @@
 #include "afm_device.cuh"
 #include "afm_f32x2.cuh"
 #include "afm_launch.h"
+#include "afm_warp.cuh"
 
 namespace afm {
 
@@ -33,6 +34,52 @@ __device__ __forceinline__ const KConst<float>& pick_k(const KConst<float>& K,
         return *sK;
     else
         return K;
+}
+
+// ---- dealt launches (a.layer > 0) ------------------------------------------
+// The swarms of an SM share its issue slots, the block that came first being
+// served first, so a launch takes as long as the SM with the most steps.
+// Measured, 304 pixels of 5120 .. 15360 steps (256 particles, two updates, two
+// blocks per SM): pulled longest first 15.4 ms; dealt by block index 13.3 ms
+// (four SMs get a pair of blocks other than b, b + 152, and those the longest
+// records); by SM 11.2 ms, with afm_warp.cuh's loop for one particle per
+// thread 10.6.
+// Placement only chooses the slot: a slot is a block's once it has set its
+// flag, and what is left over (an SM with more or fewer blocks than its
+// layers) goes to whoever asks next.
+// queue[1]: slots taken, [2]: of the last layer, [3]: SMs seen.
+__device__ __forceinline__ int take_slot(const BatchArgs& a, int slot) {
+    if (slot < 0 || slot >= a.n_pix || atomicExch(a.queue + BATCH_FLAGS + slot, 1) != 0) return -1;
+    atomicAdd(a.queue + 1, 1);
+    return slot;
+}
+
+// A block's first slot, or -1: by the SM it runs on and how many blocks came
+// there before it.
+__device__ __forceinline__ int deal(const BatchArgs& a) {
+    unsigned id;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
+    int* blocks = a.queue + 4 + id % BATCH_SMS;
+    int* index = blocks + BATCH_SMS;
+    const int l = atomicAdd(blocks, 1), full = a.n_pix / a.layer;
+    int i = -1;
+    if (l == 0) {
+        i = atomicAdd(a.queue + 3, 1);
+        atomicExch(index, i + 1);
+    }
+    if (l == full) return take_slot(a, full * a.layer + atomicAdd(a.queue + 2, 1));
+    if (l > full) return -1;
+    // the SM's first block may still be on its way to writing the index
+    for (int k = 0; k < 256 && i < 0; ++k) i = atomicAdd(index, 0) - 1;
+    return i >= 0 && i < a.layer ? take_slot(a, batch_deal(l, i, a.n_pix, a.layer)) : -1;
+}
+
+// Any slot not taken, or n_pix.
+__device__ __forceinline__ int any_left(const BatchArgs& a) {
+    if (atomicAdd(a.queue + 1, 0) >= a.n_pix) return a.n_pix;
+    for (int s = a.n_pix - 1; s >= 0; --s)
+        if (take_slot(a, s) >= 0) return s;
+    return a.n_pix;
 }
 
 }  // namespace batch_detail
@@ -68,10 +115,13 @@ __global__ void __launch_bounds__(KP == 1 ? 1024 : 512) batch_kernel(const KCons
     const KConst<float>& KK = batch_detail::pick_k<PP>(K, sK);
     const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwarps = T >> 5;
-    for (;;) {
+    for (bool first = true;; first = false) {
         __syncthreads();   // table built / previous pixel finished with shared memory
         if (tid == 0) {
-            const int sl = atomicAdd(a.queue, 1);
+            int sl = a.layer == 0 ? atomicAdd(a.queue, 1)
+                     : first      ? batch_detail::deal(a)
+                                  : -1;
+            if (sl < 0) sl = batch_detail::any_left(a);
             s_slot = sl;
             s_bad = 0;
             if (boxed && sl < a.n_pix)
@@ -162,6 +212,8 @@ __global__ void __launch_bounds__(KP == 1 ? 1024 : 512) batch_kernel(const KCons
             // pairs of particles per paired FP32 instruction where the law allows
             if constexpr (KP % 2 == 0 && M <= 4 && x2::Supported<FORCE>::value)
                 integrate_multi_x2<M, FORCE, KP>(KK, c, tab, U, n, S);
+            else if constexpr (KP == 1 && M <= 3)   // 4.5 ms a pass, 5.05 by integrate_multi
+                S[0] = integrate_warp<M, FORCE>(KK, c[0], tab, U, nullptr, 0, 0, n, false);
             else
                 integrate_multi<M, FORCE, KP>(KK, c, tab, U, n, S);
             unsigned long long key = ~0ull;
