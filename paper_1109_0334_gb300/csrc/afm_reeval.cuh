@@ -100,14 +100,17 @@ __device__ __forceinline__ double integrate64(const KConst<double>& K,
     return S;
 }
 
-// FP32 steps 0 .. n - 1 of the winner from rows in shared memory (every word
-// once); the FP64 value of the state after every AFM_SEG-th step goes to
-// Y[b][2m], b = 1 .. B - 1.  One warp's instruction stream bounds it (~130
-// per step): a step's drive terms are loaded during the step before.
+// FP32 steps of the winner from rows in shared memory (every word once); the
+// state after every AFM_SEG-th step goes to Y[b][2m], b = 1 .. B - 1, as
+// (value, compensation) for finish_start to turn into FP64: the conversions
+// (FP64 issue, 20 ns a step with one lane at work) are left to the block's
+// other threads.  One warp's instruction stream bounds it (~110 per step): a
+// step's drive terms are loaded during the step before.
+// 25 600 steps: 2.08 ms; 2.88 with the conversions in it and one step a
+// loop round.
 template <int M, int FORCE>
-__device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const KConst<double>& Kd,
-                                             const Coef<float>& cf, const float* rows, int n,
-                                             int B, double* Y) {
+__device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const Coef<float>& cf,
+                                             const float* rows, int B, double* Y) {
     constexpr int S2 = 2 * M, W = aff::Rows<M, FORCE>::words;
     const aff::LawCoef<float> c = aff::law_coef(cf);
     aff::State<float, M, aff::MODE0> s;
@@ -116,20 +119,98 @@ __device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const KCon
     const float* end = rows + (size_t)(Kf.spc2 >> 1) * W;
     float R[W];
     aff::load_row<float, M, FORCE>(Kf, row, R);
-    int b = 1, next = AFM_SEG;
-    for (int t = 0; t < n && b < B; ++t) {
-        row += W;
-        if (row == end) row = rows;
-        float Rn[W];
-        aff::load_row<float, M, FORCE>(Kf, row, Rn);
-        aff::step<float, M, FORCE, aff::MODE0>(Kf, c, R, s);
+    for (int b = 1; b < B; ++b) {   // (B - 1) AFM_SEG < n
+#pragma unroll 2
+        for (int k = 0; k < AFM_SEG; ++k) {
+            row += W;
+            if (row == end) row = rows;
+            float Rn[W];
+            aff::load_row<float, M, FORCE>(Kf, row, Rn);
+            aff::step<float, M, FORCE, aff::MODE0>(Kf, c, R, s);
 #pragma unroll
-        for (int k = 0; k < W; ++k) R[k] = Rn[k];
-        if (t + 1 == next) {
-            aff::export_state<float, M, aff::MODE0>(Kd, s, Y + (size_t)b * S2,
-                                                    Y + (size_t)b * S2 + M);
-            ++b;
-            next += AFM_SEG;
+            for (int w = 0; w < W; ++w) R[w] = Rn[w];
+        }
+        float2* y = reinterpret_cast<float2*>(Y + (size_t)b * S2);
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            y[k] = make_float2(s.q[k], k == 0 ? s.cq[0] : 0.f);
+            y[M + k] = make_float2(s.p[k], k == 0 ? s.cp[0] : 0.f);
+        }
+    }
+}
+
+// The start Y[2m] left by guess_starts as (deflections, rates) in FP64.
+template <int M>
+__device__ __forceinline__ void finish_start(const KConst<double>& Kd, double* Y) {
+    aff::State<float, M, aff::MODE0> s;
+    const float2* y = reinterpret_cast<const float2*>(Y);
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        const float2 q = y[k], v = y[M + k];
+        s.q[k] = q.x;
+        s.p[k] = v.x;
+        if (k == 0) {
+            s.cq[0] = q.y;
+            s.cp[0] = v.y;
+        }
+    }
+    double q[M], v[M];
+    aff::export_state<float, M, aff::MODE0>(Kd, s, q, v);
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        Y[k] = q[k];
+        Y[M + k] = v[k];
+    }
+}
+
+// Newton update of the segment starts, in order over the joins:
+// Znew_0 = Zold_0 (the exact initial state), Znew_{b+1} = E_b + J_b (Znew_b -
+// Zold_b); Znew may be Zold.  One warp, lanes i and 16 + i for component i:
+// the even and the odd columns of the product.  Its chain bounds it: three
+// FP64 products (for three modes), an addition and a subtraction at 64 clocks
+// of issue each and two shuffles; the operands are loaded AHEAD joins before.
+// 800 joins of three modes: 258 us, 510 with all columns in one lane and
+// operands one join ahead.
+template <int M, typename TJ>
+__device__ __forceinline__ void correct_starts(const double* Zold, double* Znew, const double* E,
+                                               const TJ* J, int B) {
+    constexpr int S2 = 2 * M, AHEAD = 4;
+    const int lane = threadIdx.x & 31, h = lane >> 4;
+    const bool store = (lane & 15) < S2 && h == 0;
+    const int i = (lane & 15) < S2 ? lane & 15 : 0;
+    double z = Zold[i], e[AHEAD], y[AHEAD];
+    // to FP64 one join ahead: at the load the conversion would wait for it, at
+    // the use the chain for the conversion
+    TJ Jr[AHEAD][M];
+    double Jd[M];
+    auto load = [&](int b, int k) {
+        b = min(b, B - 1);
+        const size_t o = (size_t)b * S2 + i;
+        e[k] = E[o];
+        y[k] = Zold[o];
+#pragma unroll
+        for (int c = 0; c < M; ++c) Jr[k][c] = J[o * S2 + 2 * c + h];
+    };
+    if (store) Znew[i] = z;
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) load(k, k);
+#pragma unroll
+    for (int c = 0; c < M; ++c) Jd[c] = (double)Jr[0][c];
+    for (int b0 = 0; b0 + 1 < B; b0 += AHEAD) {
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k) {
+            const int b = b0 + k;
+            if (b + 1 >= B) break;
+            const double dl = z - y[k];
+            double acc = h == 0 ? e[k] : 0.0;
+#pragma unroll
+            for (int c = 0; c < M; ++c)
+                acc = fma(Jd[c], __shfl_sync(0xffffffffu, dl, 2 * c + h), acc);
+#pragma unroll
+            for (int c = 0; c < M; ++c) Jd[c] = (double)Jr[(k + 1) % AHEAD][c];
+            load(b + AHEAD, k);   // reads starts that are replaced later
+            z = acc + __shfl_xor_sync(0xffffffffu, acc, 16);
+            if (store) Znew[(size_t)(b + 1) * S2 + i] = z;
         }
     }
 }

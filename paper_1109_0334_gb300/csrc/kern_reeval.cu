@@ -81,25 +81,29 @@ __global__ void __launch_bounds__(256) reeval_guess_kernel(const KConst<float> K
         if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x != 0) return;
-    *R.sumU2 = red[0];
-    ReevalWinner* w = R.win;
-    double xd[AFM_MAXD];
-    for (int d = 0; d < AFM_MAXD; ++d) xd[d] = w->x[d];
-    const Coef<double> cd = make_coef<double, double>(Kd, xd);
-    w->c[0] = cd.c0;
-    w->c[1] = cd.c1;
-    w->c[2] = cd.c2;
-    w->c[3] = cd.c3;
-    const Coef<float> c = make_coef<float, double>(Kf, xd);
     constexpr int S2 = 2 * M;
     double* Y = R.start[0];
+    if (threadIdx.x == 0) {
+        *R.sumU2 = red[0];
+        ReevalWinner* w = R.win;
+        double xd[AFM_MAXD];
+        for (int d = 0; d < AFM_MAXD; ++d) xd[d] = w->x[d];
+        const Coef<double> cd = make_coef<double, double>(Kd, xd);
+        w->c[0] = cd.c0;
+        w->c[1] = cd.c1;
+        w->c[2] = cd.c2;
+        w->c[3] = cd.c3;
+        const Coef<float> c = make_coef<float, double>(Kf, xd);
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-        Y[i] = Kd.q0[i];
-        Y[M + i] = Kd.v0[i];
+        for (int i = 0; i < M; ++i) {
+            Y[i] = Kd.q0[i];
+            Y[M + i] = Kd.v0[i];
+        }
+        guess_starts<M, FORCE>(Kf, c, tabf, R.B, Y);
     }
-    guess_starts<M, FORCE>(Kf, Kd, c, tabf, Kf.n_steps, R.B, Y);
+    __syncthreads();
+    for (int b = 1 + threadIdx.x; b < R.B; b += blockDim.x)
+        finish_start<M>(Kd, Y + (size_t)b * S2);
 }
 
 // One thread per segment b: AFM_SEG FP64 steps from Z_b -> E_b and the
@@ -180,50 +184,11 @@ __global__ void __launch_bounds__(32) reeval_pass_kernel(const KConst<double> K,
     }
 }
 
-// Newton update of the segment starts, in order over the joins:
-// Znew_0 = Zold_0 (the exact initial state), Znew_{b+1} = E_b + J_b (Znew_b -
-// Zold_b).  One warp; lane i < 2m owns state component i.
 template <int M>
 __global__ void __launch_bounds__(32) reeval_correct_kernel(const ReevalPtrs R,
                                                             const double* __restrict__ Zold,
                                                             double* __restrict__ Znew) {
-    constexpr int S2 = 2 * M;
-    const int i = threadIdx.x;
-    const bool act = i < S2;
-    const int ii = act ? i : 0;
-    double z = Zold[ii];
-    if (act) Znew[i] = z;
-    // operands of segment b are loaded one iteration ahead
-    double e = R.E[ii], y = Zold[ii], Jr[S2];
-#pragma unroll
-    for (int k = 0; k < S2; ++k) Jr[k] = R.J[(size_t)ii * S2 + k];
-    for (int b = 0; b < R.B; ++b) {
-        double en = 0.0, yn = 0.0, Jn[S2];
-#pragma unroll
-        for (int k = 0; k < S2; ++k) Jn[k] = 0.0;
-        if (b + 1 < R.B) {
-            en = R.E[(size_t)(b + 1) * S2 + ii];
-            yn = Zold[(size_t)(b + 1) * S2 + ii];
-#pragma unroll
-            for (int k = 0; k < S2; ++k) Jn[k] = R.J[((size_t)(b + 1) * S2 + ii) * S2 + k];
-        }
-        const double dl = act ? z - y : 0.0;
-        double acc0 = e, acc1 = 0.0;
-#pragma unroll
-        for (int k = 0; k < S2; ++k) {
-            const double dk = __shfl_sync(0xffffffffu, dl, k);
-            if (k & 1)
-                acc1 = fma(Jr[k], dk, acc1);
-            else
-                acc0 = fma(Jr[k], dk, acc0);
-        }
-        z = acc0 + acc1;
-        if (act) Znew[(size_t)(b + 1) * S2 + i] = z;
-        e = en;
-        y = yn;
-#pragma unroll
-        for (int k = 0; k < S2; ++k) Jr[k] = Jn[k];
-    }
+    correct_starts<M>(Zold, Znew, R.E, R.J, R.B);
 }
 
 // S_f64 = sum of the segment shares, the join check (with the sequential

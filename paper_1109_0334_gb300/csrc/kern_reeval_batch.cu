@@ -9,7 +9,7 @@
 //   sweep    (twice) one thread per segment: FP64 integration from its start
 //            with the FP32 tangent map; one warp per slot walks its joins;
 //   final    the FP64 pass from the corrected starts sums each segment's
-//            misfit share; one thread per slot adds its shares in order,
+//            misfit share; one warp per slot adds its shares,
 //            checks the joins (sequential FP64 fallback past 1e-9) and fills
 //            the result record.
 // The passes are bound by FP64 issue (~150 FP64 instructions per step in the
@@ -81,30 +81,38 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
         if (blockIdx.x == 0) aff::build_rows<double, M, FORCE>(Kd0, R.tab);
         __syncthreads();
     }
-    const int i = blockIdx.x * 32 + threadIdx.x;   // warp 0's lanes; the others built the rows
-    if (threadIdx.x >= 32 || i >= a.n_pix) return;
-    const int pix = slot_pixel(a, i);
-    const KConst<float>& Kf = pix_k<PP>(Kf0, a.pix.kf, pix);
-    const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
-    const float* tabf = PP ? a.pix.rows + (size_t)pix * a.pix.ld_rows : tabs;
-    const int n = slot_steps(a, pix);
-    double xd[AFM_MAXD];
-    for (int d = 0; d < AFM_MAXD; ++d) xd[d] = a.res[pix].x[d];
-    const Coef<double> cd = make_coef<double, double>(Kd, xd);
-    R.coef[4 * (size_t)i] = cd.c0;
-    R.coef[4 * (size_t)i + 1] = cd.c1;
-    R.coef[4 * (size_t)i + 2] = cd.c2;
-    R.coef[4 * (size_t)i + 3] = cd.c3;
-    const Coef<float> c = make_coef<float, double>(Kf, xd);
     constexpr int S2 = 2 * M;
-    double* Y = R.Z + (size_t)i * R.maxB * S2;
+    const int i = blockIdx.x * 32 + threadIdx.x;   // warp 0's lanes
+    if (threadIdx.x < 32 && i < a.n_pix) {
+        const int pix = slot_pixel(a, i);
+        const KConst<float>& Kf = pix_k<PP>(Kf0, a.pix.kf, pix);
+        const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
+        const float* tabf = PP ? a.pix.rows + (size_t)pix * a.pix.ld_rows : tabs;
+        double xd[AFM_MAXD];
+        for (int d = 0; d < AFM_MAXD; ++d) xd[d] = a.res[pix].x[d];
+        const Coef<double> cd = make_coef<double, double>(Kd, xd);
+        R.coef[4 * (size_t)i] = cd.c0;
+        R.coef[4 * (size_t)i + 1] = cd.c1;
+        R.coef[4 * (size_t)i + 2] = cd.c2;
+        R.coef[4 * (size_t)i + 3] = cd.c3;
+        const Coef<float> c = make_coef<float, double>(Kf, xd);
+        double* Y = R.Z + (size_t)i * R.maxB * S2;
 #pragma unroll
-    for (int k = 0; k < M; ++k) {
-        Y[k] = Kd.q0[k];
-        Y[M + k] = Kd.v0[k];
+        for (int k = 0; k < M; ++k) {
+            Y[k] = Kd.q0[k];
+            Y[M + k] = Kd.v0[k];
+        }
+        guess_starts<M, FORCE>(Kf, c, tabf, slot_segments(R, slot_steps(a, pix)), Y);
     }
-    const int B = slot_segments(R, n);
-    guess_starts<M, FORCE>(Kf, Kd, c, tabf, n, B, Y);
+    __syncthreads();
+    for (int w = threadIdx.x >> 5; w < 32; w += blockDim.x >> 5) {
+        const int k = blockIdx.x * 32 + w;
+        if (k >= a.n_pix) break;
+        const int pix = slot_pixel(a, k), B = slot_segments(R, slot_steps(a, pix));
+        const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
+        for (int b = 1 + (threadIdx.x & 31); b < B; b += 32)
+            finish_start<M>(Kd, R.Z + ((size_t)k * R.maxB + b) * S2);
+    }
 }
 
 // Sum of U^2 of each slot's record, one warp per slot.
@@ -195,60 +203,26 @@ __global__ void __launch_bounds__(32) rb_pass_kernel(const KConst<double> K0, co
     }
 }
 
-// Newton update of one slot's segment starts, in place, in order over its
-// joins: Z'_{b+1} = E_b + J_b (Z'_b - Z_b).  One warp per slot; lane k < 2m
-// owns state component k.
+// Newton update of every slot's segment starts, in place; one warp per slot.
 template <int M>
 __global__ void __launch_bounds__(128) rb_correct_kernel(const ReevalBatch R, const BatchArgs a) {
     constexpr int S2 = 2 * M;
     const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
-    const int k = threadIdx.x & 31;
     if (i >= a.n_pix) return;
     const int B = slot_segments(R, slot_steps(a, slot_pixel(a, i)));
-    const bool act = k < S2;
-    const int kk = act ? k : 0;
-    double* Z = R.Z + (size_t)i * R.maxB * S2;
-    const double* E = R.E + (size_t)i * R.maxB * S2;
-    const float* J = R.J + (size_t)i * R.maxB * S2 * S2;
-    double z = Z[kk];
-    double e = B > 0 ? E[kk] : 0.0, y = z;
-    float Jr[S2];
-#pragma unroll
-    for (int c = 0; c < S2; ++c) Jr[c] = B > 0 ? J[(size_t)kk * S2 + c] : 0.f;
-    for (int b = 0; b + 1 < B; ++b) {
-        // the next join's operands, read before segment b + 1's start is replaced
-        const double en = E[(size_t)(b + 1) * S2 + kk];
-        const double yn = Z[(size_t)(b + 1) * S2 + kk];
-        float Jn[S2];
-#pragma unroll
-        for (int c = 0; c < S2; ++c) Jn[c] = J[((size_t)(b + 1) * S2 + kk) * S2 + c];
-        const double dl = act ? z - y : 0.0;
-        double acc0 = e, acc1 = 0.0;
-#pragma unroll
-        for (int c = 0; c < S2; ++c) {
-            const double dc = __shfl_sync(0xffffffffu, dl, c);
-            if (c & 1)
-                acc1 = fma((double)Jr[c], dc, acc1);
-            else
-                acc0 = fma((double)Jr[c], dc, acc0);
-        }
-        z = acc0 + acc1;
-        __syncwarp();
-        if (act) Z[(size_t)(b + 1) * S2 + k] = z;
-        e = en;
-        y = yn;
-#pragma unroll
-        for (int c = 0; c < S2; ++c) Jr[c] = Jn[c];
-    }
+    const size_t g = (size_t)i * R.maxB * S2;
+    if (B > 0) correct_starts<M>(R.Z + g, R.Z + g, R.E + g, R.J + g * S2, B);
 }
 
-// Per slot: S_f64 = sum of the shares in order, the join check (sequential
-// FP64 fallback), and the result record.
+// Per slot: S_f64 = sum of the shares, the join check (sequential FP64
+// fallback), and the result record.  One warp per slot (one thread took 750 us
+// for 480 segments, a load after another).
 template <int M, int FORCE, bool PP>
 __global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, const ReevalBatch R,
                                                        const BatchArgs a) {
     constexpr int S2 = 2 * M;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
     if (i >= a.n_pix) return;
     const int pix = slot_pixel(a, i);
     const KConst<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
@@ -256,7 +230,7 @@ __global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, 
     const int B = slot_segments(R, n);
     const size_t g0 = (size_t)i * R.maxB;
     double S64 = B > 0 || n == 0 ? 0.0 : NAN, defect = 0.0;   // NaN: no room, sequential
-    for (int b = 0; b < B; ++b) {
+    for (int b = lane; b < B; b += 32) {
         S64 += R.Sb[g0 + b];
         if (b + 1 < B) {
             double mx = 0.0;
@@ -268,6 +242,12 @@ __global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, 
             defect += mx;
         }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        S64 += __shfl_xor_sync(0xffffffffu, S64, o);
+        defect += __shfl_xor_sync(0xffffffffu, defect, o);
+    }
+    if (lane != 0) return;
     int segs = B;
     if (!(defect <= kDefectTol) || !isfinite(S64)) {
         S64 = integrate64<M, FORCE, PP || aff::Table<double, M, FORCE>::compact>(
@@ -356,7 +336,7 @@ cudaError_t launch_reeval_batch(const KConst<float>& Kf, const KConst<double>& K
             if (e != cudaSuccess) return e;
             rb_pass_kernel<M, FORCE, false, PP><<<grid, 32, 0, st>>>(Kd, R, a);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            rb_final_kernel<M, FORCE, PP><<<(a.n_pix + 127) / 128, 128, 0, st>>>(Kd, R, a);
+            rb_final_kernel<M, FORCE, PP><<<cgrid, 128, 0, st>>>(Kd, R, a);
             return cudaGetLastError();
         };
         return pp ? run(std::true_type{}) : run(std::false_type{});
