@@ -175,12 +175,11 @@ def measured_peaks() -> dict:
 # (afm_launch.h, the host-side launcher declarations, is left out: adding a
 # declaration there does not change a kernel.)
 KERNEL_SOURCES = {
-    "invert_iter_kernel": ["afm_device.cuh", "afm_internal.h", "kern_invert.cu"],
-    "invert_pair_kernel": ["afm_device.cuh", "afm_internal.h", "kern_pair.cu"],
-    "invert_modes_kernel": ["afm_device.cuh", "afm_internal.h", "kern_modes.cu"],
+    "invert_iter_kernel": ["afm_device.cuh", "afm_internal.h", "afm_warp.cuh", "kern_invert.cu"],
     "fwd_kernel": ["afm_device.cuh", "afm_internal.h", "kern_forward.cu"],
     "fwd_x2_kernel": ["afm_device.cuh", "afm_internal.h", "afm_f32x2.cuh", "kern_forward.cu"],
-    "batch_kernel": ["afm_device.cuh", "afm_internal.h", "afm_f32x2.cuh", "kern_batch.cuh", "kern_batch.cu",
+    "batch_kernel": ["afm_device.cuh", "afm_internal.h", "afm_f32x2.cuh", "afm_warp.cuh",
+                     "kern_batch.cuh", "kern_batch.cu",
                      "kern_batch_dmt.cu"],
     "fe_modal_kernel": ["afm_device.cuh", "afm_internal.h", "kern_fe.cu"],
 }
@@ -904,11 +903,11 @@ def run_c2(A, W, dev, flush, peak_ops, steps=3):
            "roofline": {"bound": "alu", "achieved": ops_launch / avg_s / 1e12,
                         "peak": peak_ops / 1e12, "unit": "T FP32 lane-ops/s",
                         "frac": ops_launch / avg_s / peak_ops,
-                        "kernel": "invert_modes_kernel<3,DMT,3> (one lane per mode of a particle)",
+                        "kernel": "invert_iter_kernel<3,DMT> (one particle per lane)",
                         "ops_per_particle_step": algo_ops_per_step(m),
                         "issued_ops_per_particle_step": fp32_ops_per_step(m, spec["force"]),
                         "avg_launch_ms": avg_s * 1e3, "launches_timed": kn,
-                        "traffic": ncu_traffic("invert_modes_kernel", "c2")},
+                        "traffic": ncu_traffic("invert_iter_kernel", "c2")},
            "records_16": lm_vs_plain(A, W, "c2", dev, flush)}
     # throughput regime: one wide forward + misfit launch (262 144 particles)
     Pb = 256 * 1024

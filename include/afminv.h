@@ -394,7 +394,7 @@ afm_status afm_invert_polished(afm_ctx* ctx, const afm_problem* prob, const floa
  * n_pix), 256-aligned (the queue, the FP64 re-evaluation of every pixel's
  * winner by multiple shooting: ~250 bytes per 32-step segment of the
  * longest record and pixel, 1.6 GB for 4096 records of 51 200 steps; with
- * per-pixel problems ~6 KB per pixel of constants and drive tables). */
+ * per-pixel problems ~20 KB per pixel of constants and drive tables). */
 afm_status afm_invert_batch_workspace_size(const afm_problem* probs, int n_prob, int n_pix,
                                            size_t* bytes);
 afm_status afm_invert_batch(afm_ctx* ctx, const afm_problem* probs, int n_prob,

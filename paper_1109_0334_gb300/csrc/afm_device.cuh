@@ -294,13 +294,9 @@ __device__ __forceinline__ void kahan_add(T& x, T& c, T inc) {
     x = t;
 }
 
-// The state update of mode i: compensated or plain by comp_mode.  The plain
-// sum is the compensated one entered with c == 0 (y = inc exactly), which is
-// how kernels holding one mode per lane run it: every lane the compensated
-// form, then c masked to zero (bitwise, by the run-time KConst::cmask) where
-// the lane's mode takes plain sums.  ALL: every mode compensated (the
-// adjoint, whose gradient is more sensitive to the trajectory's rounding
-// than the misfit is).
+// The state update of mode i: compensated or plain by comp_mode.  ALL: every
+// mode compensated (the adjoint, whose gradient is more sensitive to the
+// trajectory's rounding than the misfit is).
 template <typename T, bool ALL = false>
 __device__ __forceinline__ void state_add(int i, T& x, T& c, T inc) {
     if (ALL || comp_mode<T>(i))

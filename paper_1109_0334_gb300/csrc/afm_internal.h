@@ -107,7 +107,6 @@ template <typename T>
 struct KConst {
     Affine<T> af;
     T w2[AFM_MAXM], w2lo[AFM_MAXM], wq[AFM_MAXM], gam[AFM_MAXM], tip[AFM_MAXM];
-    T cmask[AFM_MAXM];              // 1: mode i takes compensated sums (comp_mode), else 0
     T q0[AFM_MAXM], v0[AFM_MAXM];
     T Zc;
     double drive_amp, drive_phase;  // g = drive_amp * sin(2 pi j / spc2 + drive_phase)

@@ -22,9 +22,10 @@
 // or anything is non-finite, the final kernel integrates the whole record
 // once more, sequentially, in FP64.
 //
-// A 25 600-step record (three modes, DMT): the affine step (afm_affine.cuh)
-// took 1.7 ms off the ~6 ms of guess and passes in the stage form; the guess,
-// one thread's 25 600 FP32 steps, is most of what is left.
+// A 25 600-step record (three modes, DMT): guess 2.08 ms (one thread's
+// 25 600 FP32 steps, most of what is left), three passes 0.58 ms, two walks
+// over the joins 0.52 ms; with the stage form, conversions in the guess and
+// all columns of a join in one lane ~6 ms.
 #include "afm_reeval.cuh"
 
 namespace afm {
