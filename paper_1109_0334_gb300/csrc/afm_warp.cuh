@@ -283,48 +283,60 @@ __device__ __forceinline__ float integrate_warp(const KConst<float>& K, const Co
 }
 
 // The same over the deflection points (integrate_points, misfit only), any
-// lanes: the record values of a step are loaded during the step before.
-template <int M, int FORCE>
-__device__ __forceinline__ float integrate_points_warp(const KConst<float>& K,
-                                                       const Coef<float>& c, const float* tab,
-                                                       const float* __restrict__ U, int n) {
+// lanes: the record values of a step are loaded during the step before.  The
+// point count is a constant of the loop: 512 particles x 4096 steps x 3
+// points, nine launches and the re-evaluation, 5.86 ms, 8.63 with the points
+// under a uniform guard.
+template <int M, int FORCE, int NP>
+__device__ __forceinline__ float integrate_points_of(const KConst<float>& K,
+                                                     const Coef<float>& c, const float* tab,
+                                                     const float* __restrict__ U, int n) {
     const warp::Modes<M> C = warp::modes<M>(K);
     warp::State<M> s;
     warp::init<M>(K, C, tab[0], s);
     float S = 0.f, cS = 0.f;
-    const int spc2 = K.spc2, np = K.np;
+    const int spc2 = K.spc2;
     int j = 0;
     float gh = tab[1], g1 = tab[2];
-    float Ucur[AFM_MAX_POINTS];
+    float Ucur[NP];
 #pragma unroll
-    for (int k = 0; k < AFM_MAX_POINTS; ++k) Ucur[k] = (n > 0 && k < np) ? U[k] : 0.f;
+    for (int k = 0; k < NP; ++k) Ucur[k] = n > 0 ? U[k] : 0.f;
 #pragma unroll 2
     for (int t = 0; t < n; ++t) {
         j += 2;
         if (j >= spc2) j = 0;
         const float ghn = tab[j + 1], g1n = tab[j + 2];
-        float Unext[AFM_MAX_POINTS];
+        const float* Un = U + (size_t)min(t + 1, n - 1) * NP;
+        float Unext[NP];
 #pragma unroll
-        for (int k = 0; k < AFM_MAX_POINTS; ++k)
-            Unext[k] = (t + 1 < n && k < np) ? U[(size_t)(t + 1) * np + k] : 0.f;
+        for (int k = 0; k < NP; ++k) Unext[k] = Un[k];
         warp::step<M, FORCE>(C, c, gh, g1, s);
-        // unrolled to the largest point count (a uniform guard), so that the
-        // point deflections schedule alongside the step's arithmetic
 #pragma unroll
-        for (int k = 0; k < AFM_MAX_POINTS; ++k) {
-            if (k < np) {
-                float uk = __fmul_rn(K.phi[k][0], s.q[0]);
+        for (int k = 0; k < NP; ++k) {
+            float uk = __fmul_rn(K.phi[k][0], s.q[0]);
 #pragma unroll
-                for (int i = 1; i < M; ++i) uk = __fmaf_rn(K.phi[k][i], s.q[i], uk);
-                warp::misfit_add(Ucur[k], uk, S, cS);
-            }
+            for (int i = 1; i < M; ++i) uk = __fmaf_rn(K.phi[k][i], s.q[i], uk);
+            warp::misfit_add(Ucur[k], uk, S, cS);
         }
 #pragma unroll
-        for (int k = 0; k < AFM_MAX_POINTS; ++k) Ucur[k] = Unext[k];
+        for (int k = 0; k < NP; ++k) Ucur[k] = Unext[k];
         gh = ghn;
         g1 = g1n;
     }
     return S;
+}
+
+template <int M, int FORCE>
+__device__ __forceinline__ float integrate_points_warp(const KConst<float>& K,
+                                                       const Coef<float>& c, const float* tab,
+                                                       const float* __restrict__ U, int n) {
+    static_assert(AFM_MAX_POINTS == 4, "a loop per point count");
+    switch (K.np) {
+        case 1: return integrate_points_of<M, FORCE, 1>(K, c, tab, U, n);
+        case 2: return integrate_points_of<M, FORCE, 2>(K, c, tab, U, n);
+        case 3: return integrate_points_of<M, FORCE, 3>(K, c, tab, U, n);
+        default: return integrate_points_of<M, FORCE, 4>(K, c, tab, U, n);
+    }
 }
 
 }  // namespace afm
