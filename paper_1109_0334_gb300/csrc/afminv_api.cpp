@@ -20,6 +20,7 @@ using afm::KConst;
 
 #include <map>
 #include <tuple>
+#include <functional>
 #include <vector>
 
 // One instantiated launch graph of afm_invert_batch and the argument bytes it
@@ -1035,7 +1036,8 @@ void append_bytes(std::vector<unsigned char>& v, const T& x) {
 // of pixels for each particles-per-thread choice and keeps the one with the
 // lowest estimated batch time (the wave's time x the waves the batch needs).
 afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst& pc,
-                      const afm::BatchArgs& a, cudaStream_t s, int* kp_out, int* occ_out) {
+                      const afm::BatchArgs& a, bool selected, cudaStream_t s, int* kp_out,
+                      int* occ_out) {
     const bool pp = a.pix.kf != nullptr;
     const auto key = std::make_tuple(Kf.m, Kf.force, pc.P, pc.D, Kf.spc2, (int)pp);
     auto it = ctx->batch_kp.find(key);
@@ -1044,6 +1046,17 @@ afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst
         AFM_CUDA(afm::batch_occupancy(Kf.m, Kf.force, *kp_out, pc.P, pc.D, Kf.spc2, pp, occ_out),
                  "batch occupancy");
         return AFM_OK;
+    }
+    // record steps of the slots, in slot order (not of a caller's selection)
+    std::vector<int64_t> steps;
+    if (!selected) {
+        std::vector<int64_t> off((size_t)a.n_pix + 1);
+        AFM_CUDA(cudaMemcpyAsync(off.data(), a.off, sizeof(int64_t) * off.size(),
+                                 cudaMemcpyDeviceToHost, s),
+                 "record offsets");
+        AFM_CUDA(cudaStreamSynchronize(s), "record offsets");
+        for (int i = 0; i < a.n_pix; ++i) steps.push_back(off[i + 1] - off[i]);
+        if (a.order) std::sort(steps.begin(), steps.end(), std::greater<int64_t>());
     }
     float best_ms = 1e30f;
     int best_kp = 0, best_occ = 0;
@@ -1073,9 +1086,20 @@ afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst
         float ms = 0.f;
         AFM_CUDA(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
         // the probe is one wave of the resident pixels (num_sms x occ, which
-        // differs between candidates): estimate the whole batch as that
-        // wave's time per resident pixel times the pixels
-        ms *= std::max(1.0f, (float)a.n_pix / (float)pa.n_pix);
+        // differs between candidates), the longest ones: estimate the whole
+        // batch as that wave's time per record step times the steps (per
+        // pixel the candidate with more resident pixels, shorter ones among
+        // them, looked 6 % better on 4096 pixels of 20 to 200 cycles)
+        double share = (double)a.n_pix / (double)pa.n_pix;
+        if (!selected) {
+            double all = 0.0, probed = 0.0;
+            for (int i = 0; i < a.n_pix; ++i) {
+                all += (double)steps[i];
+                if (i < pa.n_pix) probed += (double)steps[i];
+            }
+            if (probed > 0.0) share = all / probed;
+        }
+        ms *= (float)std::max(1.0, share);
         if (ms < best_ms) {
             best_ms = ms;
             best_kp = kp;
@@ -1930,7 +1954,7 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
         if (occ < 1) return fail(AFM_ERR_UNSUPPORTED, "batch kernel does not fit (P = %d)", pc.P);
     } else if (want != 0) {
         return fail(AFM_ERR_INVALID_ARG, "particles_per_thread must be 0 (tune), 1, 2 or 4");
-    } else if ((st = batch_tune(ctx, B.Kf, pc, a, s, &kp, &occ))) {
+    } else if ((st = batch_tune(ctx, B.Kf, pc, a, select != nullptr, s, &kp, &occ))) {
         return st;
     }
     B.kp = kp;
