@@ -1,6 +1,7 @@
 // kern_batch.cu -- many independent pixel inversions (IP of Sec. 2.3, one per
 // pixel of an image scan) in one persistent launch.  Each block pulls pixels
-// from an atomic queue (longest record first) and runs that pixel's whole
+// from an atomic queue (longest record first), or is dealt one where every
+// pixel has a resident block (kern_batch.cuh), and runs that pixel's whole
 // particle swarm (Sec. 3.4, Eq. 8) on chip: positions, velocities and
 // personal bests in shared memory, the global best reduced with warp shuffles
 // and one shared-memory pass, every swarm evaluation the fused RK4 (Eq. 2) +

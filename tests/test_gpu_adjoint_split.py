@@ -1,7 +1,7 @@
-"""The adjoint of few particles on one record (segments at once,
-joined by their maps of the adjoint state): S and G of it, and of the one-kernel form which takes over for
-larger batches, against the oracle's complex
-step.  Step counts around the 32-step segments."""
+"""The adjoint of few particles on one record (segments at once, joined by
+their maps of the adjoint state): S and G of it, and of the one-kernel form
+which takes over for larger batches, against the oracle's complex step.  Step
+counts around the 32-step segments."""
 import numpy as np
 import pytest
 
