@@ -132,6 +132,32 @@ __device__ __forceinline__ T fe_sum(const T* wp) {
     return s[0];
 }
 
+// The tip deflection of a particle from its lanes' slots, the same bits for 4
+// and 8 lanes: a 4-lane lane's even slots are the modes of one lane of eight
+// and its odd slots those of the lane four further on, so it sums the two
+// apart and adds them where the 8-lane butterfly exchanges them.  A
+// particle's misfit then does not depend on how many share its launch (a
+// swarm split over processes is the whole swarm bit for bit).
+template <typename T, int FEL>
+__device__ __forceinline__ T fe_tip(const T (&zp)[FEN / FEL]) {
+    constexpr int FEM = FEN / FEL;
+    T t;
+    if constexpr (FEL == 4) {
+        T even[FEM / 2], odd[FEM / 2];
+#pragma unroll
+        for (int k = 0; k < FEM / 2; ++k) {
+            even[k] = zp[2 * k];
+            odd[k] = zp[2 * k + 1];
+        }
+        t = fe_sum<T, FEM / 2>(even) + fe_sum<T, FEM / 2>(odd);
+    } else {
+        t = fe_sum<T, FEM>(zp);
+    }
+#pragma unroll
+    for (int o = FEL / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
 // z = base + cz F(Zc + z) by Newton from z = base + cz Fguess.
 template <int FORCE, typename T>
 __device__ __forceinline__ T fe_newton(const Coef<T>& c, T Zc, T base, T cz, T Fguess, int iters,
@@ -287,9 +313,7 @@ __global__ void __launch_bounds__(FE_THREADS, FEL == 4 ? FE_MIN_BLOCKS4 : FE_MIN
             incs[j] = inc;
             zps[j] = fe_comp<T, FEL>(j) ? z[j] + ((dz[j] + inc) - cz[k]) : z[j] + inc;
         }
-        T tsum = fe_sum<T, FEM>(zps);
-#pragma unroll
-        for (int o = FEL / 2; o > 0; o >>= 1) tsum += __shfl_xor_sync(0xffffffffu, tsum, o);
+        const T tsum = fe_tip<T, FEL>(zps);
         T Fp;
         fe_newton<FORCE, T>(cfc, Zc, tsum, ctip, sizeof(T) == 8 ? Fn : (T)0, newton_it, Fp);
         // compensated updates of both the increment and the modal coordinate
