@@ -306,9 +306,17 @@ afm_status afm_invert(afm_ctx* ctx, const afm_problem* prob, const float* U,
  * the reverse sweep.  The adjoint compensates the state update of every
  * mode (afm_forward_batch: the lowest mode only), so its S agrees with
  * afm_forward_batch's within 1e-4 relative, not bit for bit.  The Kahan
- * compensation is treated as exact addition.  workspace: device,
- * >= afm_adjoint_workspace_size (the checkpoints: ceil(n_steps/32) x 4 x
- * modes x P floats). */
+ * compensation is treated as exact addition.
+ * Few particles are taken in 32-step segments at once (the step as an affine
+ * map, the segments' maps of the adjoint state joined in FP64), more in one
+ * kernel; the two round differently, so S and dS_dx of a particle may change
+ * in their last digits with P, n_steps and workspace_bytes.
+ * workspace: device.  The checkpoints are enough, C = ceil(n_steps/32) x 4 x
+ * M x P floats rounded up to 256 bytes, M = 1, 3 or (any other n_modes) 8;
+ * the segments at once also take their records, at most 256 MB, and run
+ * where workspace_bytes has room for them.  afm_adjoint_workspace_size gives
+ * the room for both; it does not fall as P or n_steps grows, so one buffer of
+ * the largest batch's size serves the smaller ones. */
 afm_status afm_adjoint_workspace_size(const afm_problem* prob, int P, size_t* bytes);
 afm_status afm_adjoint(afm_ctx* ctx, const afm_problem* prob, const float* x, int P,
                        const float* U, float* S, float* dS_dx, void* workspace,

@@ -403,15 +403,23 @@ def adjoint_workspace_size(prob: Problem, P: int) -> int:
     return int(n.value)
 
 
+def _adjoint_checkpoint_bytes(prob: Problem, P: int) -> int:
+    """The least workspace that afm_adjoint takes."""
+    m = 1 if prob.model == _MODEL["point_mass"] else int(prob.n_modes)
+    nbytes = 16 * -(-int(prob.n_steps) // 32) * (m if m in (1, 3) else MAX_MODES) * P
+    return -(-nbytes // 256) * 256
+
+
 def adjoint(prob: Problem, x, U, workspace=None, stream=None):
     """Misfit S [P] and its gradient dS/dx [D, P] for x float32 CUDA [D, P]
-    (discrete adjoint of the FP32 RK4 + compensated misfit)."""
+    (discrete adjoint of the FP32 RK4 + compensated misfit).  workspace: a
+    uint8 CUDA tensor of adjoint_workspace_size, or one of at least the
+    checkpoints' size (slower for few particles)."""
     import torch
     D, P = int(x.shape[0]), int(x.shape[1])
     dev = x.device
-    nbytes = adjoint_workspace_size(prob, P)
-    if workspace is None or workspace.numel() < nbytes:
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=dev)
+    if workspace is None or workspace.numel() < _adjoint_checkpoint_bytes(prob, P):
+        workspace = torch.empty(adjoint_workspace_size(prob, P), dtype=torch.uint8, device=dev)
     S = torch.empty(P, dtype=torch.float32, device=dev)
     G = torch.empty((D, P), dtype=torch.float32, device=dev)
     _check(lib().afm_adjoint(context(dev.index), C.byref(prob), _ptr(x), P, _ptr(U), _ptr(S),

@@ -114,10 +114,11 @@ cudaError_t launch_batch(const KConst<float>& K, const PsoConst& pc, const Batch
 // record U + off[pix] of length off[pix+1] - off[pix] <= K.n_steps; records
 // longer than K.n_steps give S = inf and a zero gradient.
 size_t adjoint_ckpt_floats(int m, int n_steps, int P);
-// One record for all particles, in segments where they are few
-// (kern_adjoint.cu); ws: adjoint_ws_floats.
+// One record for all particles, in segments where they are few and ws has room
+// (kern_adjoint.cu); ws_bytes: at least the checkpoints, adjoint_ws_floats for
+// the segments.
 cudaError_t launch_adjoint_split(const KConst<float>& K, const float* x, int P, const float* U,
-                                 float* S, float* G, float* ws, cudaStream_t st);
+                                 float* S, float* G, float* ws, size_t ws_bytes, cudaStream_t st);
 size_t adjoint_ws_floats(int m, int force, int n_steps, int P);
 cudaError_t launch_adjoint(const KConst<float>& K, const float* x, int P, const float* U, float* S,
                            float* G, float* ckpt, cudaStream_t st, const int64_t* off = nullptr,

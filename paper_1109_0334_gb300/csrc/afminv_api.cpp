@@ -1563,15 +1563,18 @@ afm_status afm_adjoint(afm_ctx* ctx, const afm_problem* prob, const float* x, in
     if (P < 1 || prob->n_free < 1) return fail(AFM_ERR_INVALID_ARG, "P >= 1 and n_free >= 1 needed");
     if (!x || !U || !S || !dS_dx || !workspace)
         return fail(AFM_ERR_INVALID_ARG, "NULL x, U, S, dS_dx or workspace");
-    size_t need = 0;
-    if ((st = afm_adjoint_workspace_size(prob, P, &need))) return st;
+    // the checkpoints; without room for the segments' records the one-kernel
+    // form runs
+    const size_t need = align256(
+        sizeof(float) * afm::adjoint_ckpt_floats(problem_modes(*prob), prob->n_steps, P));
     if (workspace_bytes < need)
         return fail(AFM_ERR_INVALID_ARG, "workspace %zu bytes < %zu needed", workspace_bytes, need);
     KConst<float> K;
     fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AFM_CUDA(timed_launch(ctx, s, [&] {
-                 return afm::launch_adjoint_split(K, x, P, U, S, dS_dx, static_cast<float*>(workspace), s);
+                 return afm::launch_adjoint_split(K, x, P, U, S, dS_dx, static_cast<float*>(workspace),
+                                                  workspace_bytes, s);
              }),
              "adjoint kernel");
     return AFM_OK;

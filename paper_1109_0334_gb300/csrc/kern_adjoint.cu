@@ -43,6 +43,7 @@
 // one kernel; 200 us of it the forward solve (78 ns a step), the chain left.
 // With the adjoint state taken back serially, one lane a particle: 307 us for
 // that pass alone.
+#include <algorithm>
 #include <type_traits>
 
 #include "afm_affine.cuh"
@@ -349,9 +350,13 @@ size_t split_floats(int M, bool rate, int n_steps, int P) {
 // Measured at 1280 steps, split / one kernel: 3 modes, 2048 particles
 // 377 / 675 us, 4864 612 / 677; 1 mode, 4864 412 / 482; 8 modes, 2200
 // 995 / 1205.  Its records stay within 256 MB.
+constexpr size_t SPLIT_FLOATS = 64u << 20;
+
+int split_max_particles(int M) { return 40000 / (2 * M + 2); }
+
 bool adj_split(int M, int force, int n_steps, int P) {
-    return (long long)P * (2 * M + 2) <= 40000 &&
-           split_floats(M, rate_law(force), n_steps, P) <= (64u << 20);
+    return P <= split_max_particles(M) &&
+           split_floats(M, rate_law(force), n_steps, P) <= SPLIT_FLOATS;
 }
 
 // One step of the adjoint state back in time: the cotangents lq, lp of the
@@ -741,17 +746,23 @@ size_t adjoint_ckpt_floats(int m, int n_steps, int P) {
     return (size_t)((n_steps + SEG - 1) / SEG) * 4 * tmodes(m) * P;
 }
 
+// The checkpoints with room for the split form's records at P particles and
+// below: it grows with P and with n_steps, so a buffer of a larger batch's or a
+// longer record's size serves a smaller one's split form too.
 size_t adjoint_ws_floats(int m, int force, int n_steps, int P) {
-    const int M = tmodes(m);
-    return adjoint_ckpt_floats(m, n_steps, P) +
-           (adj_split(M, force, n_steps, P) ? split_floats(M, rate_law(force), n_steps, P) : 0);
+    const int M = tmodes(m), Ps = std::min(P, split_max_particles(M));
+    const size_t split = adjoint_ckpt_floats(m, n_steps, Ps) +
+                         std::min(split_floats(M, rate_law(force), n_steps, Ps), SPLIT_FLOATS);
+    return std::max(adjoint_ckpt_floats(m, n_steps, P), split);
 }
 
 cudaError_t launch_adjoint_split(const KConst<float>& K, const float* x, int P,
                                         const float* U, float* S, float* G, float* ckpt,
-                                        cudaStream_t st) {
-    if (!adj_split(tmodes(K.m), K.force, K.n_steps, P) ||
-        reinterpret_cast<uintptr_t>(ckpt) % 16 != 0)
+                                        size_t ws_bytes, cudaStream_t st) {
+    const int Mt = tmodes(K.m);
+    if (!adj_split(Mt, K.force, K.n_steps, P) || reinterpret_cast<uintptr_t>(ckpt) % 16 != 0 ||
+        ws_bytes / sizeof(float) < adjoint_ckpt_floats(K.m, K.n_steps, P) +
+                                       split_floats(Mt, rate_law(K.force), K.n_steps, P))
         return launch_adjoint(K, x, P, U, S, G, ckpt, st);
     const int nseg = (K.n_steps + SEG - 1) / SEG;
     const int ppb = warp::per_block(P), blocks = (P + ppb - 1) / ppb;
