@@ -345,17 +345,30 @@ size_t split_floats(int M, bool rate, int n_steps, int P) {
     return ((rate ? 9 : 5) * (size_t)n_steps + (4 + 2 * map_words(M)) * seg) * P;
 }
 
-// The maps take 2 M + 1 columns and the way back one more, so the split form
-// pays while P (2 M + 2) lanes' work is below one warp's serial time.
-// Measured at 1280 steps, split / one kernel: 3 modes, 2048 particles
-// 377 / 675 us, 4864 612 / 677; 1 mode, 4864 412 / 482; 8 modes, 2200
-// 995 / 1205.  Its records stay within 256 MB.
+// Where the split form pays.  It saves ~0.4 us of one warp's serial time a
+// step, and costs five more launches (~55 us) and the work of the maps' 2 M + 1
+// columns and the way back, ~0.05 ns x P a step and column, which the one
+// kernel's idle SMs would not have done.  Measured, one kernel / split:
+//   few particles (32): 160 steps 0.96 .. 1.27, 200 1.08 .. 1.45, 256 1.2 ..
+//     1.6, 512 1.7 .. 2.4, 2500 3.1 .. 4.0
+//   break-even particles at 256 / 512 / 1000 steps: 1 mode (DMT) 1750 / 3800 /
+//     5800, 3 modes (DMT + KV, spring-damper) 2400 / 3300 / 4000, 8 modes
+//     (spring-damper) 1800 / 2100 / past 2222
+//   its blocks build their drive rows, which shows past 512 phases: at 1280
+//     steps 3 modes break even at 4000 particles with 1024 phases and 2700 with
+//     2048, 8 modes (spring-damper) past 1700 and at 1400
+// The lines below stay within those: 0.99 at their worst, where the start of
+// the range meets one mode.
+long long split_max_particles(int M, int n_steps) {
+    const long long most = M == 1 ? 6000 : (M == 3 ? 4000 : 1700);
+    return std::max(0ll, std::min({most, 12 * (n_steps - 180ll), 2000 + 2ll * n_steps}));
+}
+
+// Its records stay within 256 MB.
 constexpr size_t SPLIT_FLOATS = 64u << 20;
 
-int split_max_particles(int M) { return 40000 / (2 * M + 2); }
-
-bool adj_split(int M, int force, int n_steps, int P) {
-    return P <= split_max_particles(M) &&
+bool adj_split(int M, int force, int n_steps, int spc, int P) {
+    return P <= split_max_particles(M, n_steps) && (long long)P * spc <= (M <= 3 ? 4000000 : 1500000) &&
            split_floats(M, rate_law(force), n_steps, P) <= SPLIT_FLOATS;
 }
 
@@ -750,7 +763,8 @@ size_t adjoint_ckpt_floats(int m, int n_steps, int P) {
 // below: it grows with P and with n_steps, so a buffer of a larger batch's or a
 // longer record's size serves a smaller one's split form too.
 size_t adjoint_ws_floats(int m, int force, int n_steps, int P) {
-    const int M = tmodes(m), Ps = std::min(P, split_max_particles(M));
+    const int M = tmodes(m);
+    const int Ps = (int)std::min((long long)P, split_max_particles(M, n_steps));
     const size_t split = adjoint_ckpt_floats(m, n_steps, Ps) +
                          std::min(split_floats(M, rate_law(force), n_steps, Ps), SPLIT_FLOATS);
     return std::max(adjoint_ckpt_floats(m, n_steps, P), split);
@@ -760,7 +774,7 @@ cudaError_t launch_adjoint_split(const KConst<float>& K, const float* x, int P,
                                         const float* U, float* S, float* G, float* ckpt,
                                         size_t ws_bytes, cudaStream_t st) {
     const int Mt = tmodes(K.m);
-    if (!adj_split(Mt, K.force, K.n_steps, P) || reinterpret_cast<uintptr_t>(ckpt) % 16 != 0 ||
+    if (!adj_split(Mt, K.force, K.n_steps, K.spc2 / 2, P) || reinterpret_cast<uintptr_t>(ckpt) % 16 != 0 ||
         ws_bytes / sizeof(float) < adjoint_ckpt_floats(K.m, K.n_steps, P) +
                                        split_floats(Mt, rate_law(K.force), K.n_steps, P))
         return launch_adjoint(K, x, P, U, S, G, ckpt, st);
