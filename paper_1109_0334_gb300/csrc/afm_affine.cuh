@@ -118,7 +118,7 @@ struct Table {
 // The drive terms of every phase of the period, evaluated in FP64 by the
 // block's threads.
 template <typename T, int M, int FORCE>
-__device__ __forceinline__ void build_rows(const KConst<T>& K, T* tab) {
+__device__ __forceinline__ void build_rows(const KAffine<T>& K, T* tab) {
     using R = Rows<M, FORCE>;
     using Tb = Table<T, M, FORCE>;
     const int spc = K.spc2 >> 1;
@@ -140,7 +140,7 @@ __device__ __forceinline__ void build_rows(const KConst<T>& K, T* tab) {
 
 // The terms of a phase from its sine and cosine.
 template <int M, int FORCE>
-__device__ __forceinline__ void phase_terms(const KConst<double>& K, double s, double c,
+__device__ __forceinline__ void phase_terms(const KAffine<double>& K, double s, double c,
                                             double (&r)[Rows<M, FORCE>::words]) {
 #pragma unroll
     for (int k = 0; k < Rows<M, FORCE>::words; ++k)
@@ -149,7 +149,7 @@ __device__ __forceinline__ void phase_terms(const KConst<double>& K, double s, d
 
 // One row into registers, 16 bytes per load.
 template <typename T, int M, int FORCE>
-__device__ __forceinline__ void load_row(const KConst<T>& K, const T* __restrict__ row,
+__device__ __forceinline__ void load_row(const KAffine<T>& K, const T* __restrict__ row,
                                          T (&r)[Rows<M, FORCE>::words]) {
     constexpr int WORDS = Rows<M, FORCE>::words;
     static_assert(WORDS % 4 == 0, "16-byte rows");
@@ -198,7 +198,7 @@ __device__ __forceinline__ V sum_tail(const V* a) {   // a[1] + a[2] + ...
 }
 
 template <typename V, int M, int COMP, typename T>
-__device__ __forceinline__ void init(const KConst<T>& K, State<V, M, COMP>& s) {
+__device__ __forceinline__ void init(const KAffine<T>& K, State<V, M, COMP>& s) {
 #pragma unroll
     for (int i = 0; i < M; ++i) {
         s.q[i] = K.q0[i];
@@ -240,7 +240,7 @@ struct Stages {
 };
 
 template <typename V, int M, int FORCE, int COMP, typename T>
-__device__ __forceinline__ void stages(const KConst<T>& K, const LawCoef<V>& c, const V* R,
+__device__ __forceinline__ void stages(const KAffine<T>& K, const LawCoef<V>& c, const V* R,
                                        const State<V, M, COMP>& s, Stages<V>& g) {
     const Affine<T>& A = K.af;
     constexpr bool rate = UsesRate<FORCE>::value;
@@ -305,7 +305,7 @@ __device__ __forceinline__ void stages(const KConst<T>& K, const LawCoef<V>& c, 
 
 // The step's increments from its four stage forces.
 template <typename V, int M, int COMP, typename T>
-__device__ __forceinline__ void advance(const KConst<T>& K, const V* R, const V* F,
+__device__ __forceinline__ void advance(const KAffine<T>& K, const V* R, const V* F,
                                         State<V, M, COMP>& s) {
     const Affine<T>& A = K.af;
     {
@@ -347,7 +347,7 @@ __device__ __forceinline__ void advance(const KConst<T>& K, const V* R, const V*
 }
 
 template <typename V, int M, int FORCE, int COMP, typename T>
-__device__ __forceinline__ void step(const KConst<T>& K, const LawCoef<V>& c, const V* R,
+__device__ __forceinline__ void step(const KAffine<T>& K, const LawCoef<V>& c, const V* R,
                                      State<V, M, COMP>& s) {
     Stages<V> g;
     stages<V, M, FORCE, COMP>(K, c, R, s, g);
@@ -367,7 +367,7 @@ __device__ __forceinline__ void misfit_add(V U, V u, V& S, V& cS) {
 // Deflection at point k of the cantilever (K.phi), in the order of tip(), so
 // that a point at the tip gives the tip's bits.
 template <typename V, int M, int COMP, typename T>
-__device__ __forceinline__ V point_defl(const KConst<T>& K, int k, const State<V, M, COMP>& s) {
+__device__ __forceinline__ V point_defl(const KAffine<T>& K, int k, const State<V, M, COMP>& s) {
     if constexpr (M > 1) {
         V t = mul(K.phi[k][1], s.q[1]);
 #pragma unroll
@@ -380,7 +380,7 @@ __device__ __forceinline__ V point_defl(const KConst<T>& K, int k, const State<V
 
 // The state as (deflections, rates per tau) in FP64, compensations included.
 template <typename T, int M, int COMP>
-__device__ __forceinline__ void export_state(const KConst<double>& K, const State<T, M, COMP>& s,
+__device__ __forceinline__ void export_state(const KAffine<double>& K, const State<T, M, COMP>& s,
                                              double* q, double* v) {
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -393,7 +393,7 @@ __device__ __forceinline__ void export_state(const KConst<double>& K, const Stat
 
 // ... and from them (uncompensated).
 template <int M>
-__device__ __forceinline__ void import_state(const KConst<double>& K, const double* q,
+__device__ __forceinline__ void import_state(const KAffine<double>& K, const double* q,
                                              const double* v, State<double, M, NONE>& s) {
 #pragma unroll
     for (int i = 0; i < M; ++i) {

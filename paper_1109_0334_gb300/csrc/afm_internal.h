@@ -105,7 +105,11 @@ AFM_HD constexpr bool rate_law(int force) { return force == 2 || force == 4; }
 // double), filled on the host by the per-problem set-up.
 template <typename T>
 struct KConst {
-    Affine<T> af;
+    // The arrays start 8 bytes past a 16-byte boundary, here and in KAffine: on
+    // one, the compiler reads them 16 bytes at a time into more registers, and
+    // the eight-mode kernels were slower (DMT, 19 457 particles x 512 steps 220
+    // us, 211 so; Hooke's sensitivities, 512 x 512 steps, 212 us, 196 so).
+    double skew;
     T w2[AFM_MAXM], w2lo[AFM_MAXM], wq[AFM_MAXM], gam[AFM_MAXM], tip[AFM_MAXM];
     T q0[AFM_MAXM], v0[AFM_MAXM];
     T Zc;
@@ -119,6 +123,23 @@ struct KConst {
     int np;                         // deflection points (kern_points.cu), 0: the tip
     T phi[4][AFM_MAXM];             // tip-normalised mode shapes at the points
 };
+
+// The constants with the step's affine map, for the kernels that run it.  The
+// stage-form kernels (every FP32 solve and swarm) take KConst alone: the map is
+// two thirds of the words, and forming it costs the host 2 of a call's 11 us for
+// three modes in FP32, 6 of 22 for eight (10 and 30 us on an x86 core), once per
+// pixel where the pixels' problems differ.
+template <typename T>
+struct AffineFirst {
+    Affine<T> af;
+    double skew[3];   // see KConst
+};
+template <typename T>
+struct KAffine : AffineFirst<T>, KConst<T> {};
+// no padding between or after: the bytes are part of a launch graph's key
+static_assert(sizeof(KAffine<float>) == sizeof(KConst<float>) + sizeof(Affine<float>) + 24 &&
+                  sizeof(KAffine<double>) == sizeof(KConst<double>) + sizeof(Affine<double>) + 24,
+              "KAffine has padding");
 
 // Finite-element cantilever (cubic Hermite elements, clamped node removed)
 // advanced by Newmark's average-acceleration scheme (beta = 1/4, gamma = 1/2)

@@ -34,7 +34,7 @@ struct PsoConst {
 cudaError_t launch_forward_f32(const KConst<float>& K, const float* x, int P, float* defl,
                                const float* U, float* S, int* flags, cudaStream_t st,
                                int lanes = 0);
-cudaError_t launch_forward_f64(const KConst<double>& K, const double* x, int P, double* defl,
+cudaError_t launch_forward_f64(const KAffine<double>& K, const double* x, int P, double* defl,
                                const double* U, double* S, int* flags, cudaStream_t st);
 // standalone misfit of a time-major deflection array
 cudaError_t launch_misfit(const float* defl, const float* U, int N, int P, float* S, int num_sms,
@@ -50,8 +50,8 @@ cudaError_t launch_synth(const KConst<float>& K, const double* x_truth, int n_pi
 // and the drive terms of the affine step: FP32 rows and the FP64 sine and
 // cosine of each phase (tab64).  kf == nullptr: every pixel uses the launch's constants.
 struct PixConst {
-    const KConst<float>* kf;    // [n_pix]
-    const KConst<double>* kd;   // [n_pix]
+    const KAffine<float>* kf;   // [n_pix]
+    const KAffine<double>* kd;  // [n_pix]
     const double* tab64;        // [n_pix][ld64]
     const float* tab32;         // [n_pix][ld]
     const float* rows;          // [n_pix][ld_rows]
@@ -114,11 +114,13 @@ cudaError_t launch_batch(const KConst<float>& K, const PsoConst& pc, const Batch
 // record U + off[pix] of length off[pix+1] - off[pix] <= K.n_steps; records
 // longer than K.n_steps give S = inf and a zero gradient.
 size_t adjoint_ckpt_floats(int m, int n_steps, int P);
-// One record for all particles, in segments where they are few and ws has room
-// (kern_adjoint.cu); ws_bytes: at least the checkpoints, adjoint_ws_floats for
-// the segments.
-cudaError_t launch_adjoint_split(const KConst<float>& K, const float* x, int P, const float* U,
-                                 float* S, float* G, float* ws, size_t ws_bytes, cudaStream_t st);
+// One record for all particles, its segments at once (kern_adjoint.cu): for
+// batches and workspaces that adjoint_runs_split accepts; adjoint_ws_floats has
+// room for it wherever it pays.
+bool adjoint_runs_split(int m, int force, int n_steps, int spc, int P, const void* ws,
+                        size_t ws_bytes);
+cudaError_t launch_adjoint_split(const KAffine<float>& K, const float* x, int P, const float* U,
+                                 float* S, float* G, float* ws, cudaStream_t st);
 size_t adjoint_ws_floats(int m, int force, int n_steps, int P);
 cudaError_t launch_adjoint(const KConst<float>& K, const float* x, int P, const float* U, float* S,
                            float* G, float* ckpt, cudaStream_t st, const int64_t* off = nullptr,
@@ -128,14 +130,14 @@ cudaError_t launch_adjoint(const KConst<float>& K, const float* x, int P, const 
 // [P][D][D], b [P][D]; ragged form as launch_adjoint), damped trial points,
 // choice of the best trial point
 // (pix: per-pixel constants of the ragged form, pix.kf == nullptr: K for all)
-cudaError_t launch_sens(const KConst<float>& K, const float* x, int P, const float* U, float* S,
+cudaError_t launch_sens(const KAffine<float>& K, const float* x, int P, const float* U, float* S,
                         double* H, double* b, cudaStream_t st, const int64_t* off = nullptr,
                         const int* order = nullptr, int per_slot = 1,
                         const PixConst& pix = PixConst{});
 // the same pass with one lane per parameter direction (kern_lm_lanes.cu);
 // launch_sens uses it when P x lanes fits one warp per SM sub-partition
 bool sens_lanes_preferred(int P, int D);
-cudaError_t launch_sens_lanes(const KConst<float>& K, const float* x, int P, const float* U,
+cudaError_t launch_sens_lanes(const KAffine<float>& K, const float* x, int P, const float* U,
                               float* S, double* H, double* b, cudaStream_t st, const int64_t* off,
                               const int* order, int per_slot);
 cudaError_t launch_lm_cand(int D, int K, int J, const float* x, const double* H, const double* b,
@@ -259,7 +261,7 @@ void reeval_batch_carve(void* base, int m, int force, int n_steps, int spc, int 
                         ReevalBatch* R);
 // fills each slot's result record (S_f64, J_rel, theta, status, defect,
 // segments) from the parameters already in it
-cudaError_t launch_reeval_batch(const KConst<float>& Kf, const KConst<double>& Kd,
+cudaError_t launch_reeval_batch(const KAffine<float>& Kf, const KAffine<double>& Kd,
                                 const ReevalBatch& R, const BatchArgs& a, cudaStream_t st);
 bool reeval_supported(int m, int n_steps);
 size_t reeval_bytes(int m, int n_steps, int spc);
@@ -268,7 +270,7 @@ cudaError_t launch_reeval_pick_swarm(const PsoConst& pc, const SwarmPtrs& sw, fl
                                      ReevalWinner* w, cudaStream_t st);
 cudaError_t launch_reeval_pick_min(int D, int Kn, const float* x, const float* S, const int* idx,
                                    ReevalWinner* w, cudaStream_t st);
-cudaError_t launch_reeval(const KConst<float>& Kf, const KConst<double>& Kd, const ReevalPtrs& R,
+cudaError_t launch_reeval(const KAffine<float>& Kf, const KAffine<double>& Kd, const ReevalPtrs& R,
                           const float* U, int iters, const int* flags, void* result,
                           cudaStream_t st);
 

@@ -47,7 +47,7 @@ cudaError_t dispatch_m13(int m, int force, F&& f) {
 // force slopes of each stage go to rec[k * 32], k = 2 * stage (+1 for the rate
 // slope).
 template <int M, int FORCE, bool REC>
-__device__ __forceinline__ void step64(const KConst<double>& K, const aff::LawCoef<double>& c,
+__device__ __forceinline__ void step64(const KAffine<double>& K, const aff::LawCoef<double>& c,
                                        const Coef<float>& cf, const double* R,
                                        aff::State<double, M, aff::NONE>& s, float* rec) {
     aff::Stages<double> g;
@@ -67,7 +67,7 @@ __device__ __forceinline__ void step64(const KConst<double>& K, const aff::LawCo
 // Drive terms of phase j.  COMPACT: tab holds the sine and cosine of each
 // phase (2 spc doubles), else the rows of build_rows.
 template <int M, int FORCE, bool COMPACT>
-__device__ __forceinline__ void drive_terms(const KConst<double>& K, const double* tab, int j,
+__device__ __forceinline__ void drive_terms(const KAffine<double>& K, const double* tab, int j,
                                             double (&R)[aff::Rows<M, FORCE>::words]) {
     if constexpr (COMPACT)
         aff::phase_terms<M, FORCE>(K, tab[2 * j], tab[2 * j + 1], R);
@@ -77,7 +77,7 @@ __device__ __forceinline__ void drive_terms(const KConst<double>& K, const doubl
 
 // The whole record by one thread: the fallback of both re-evaluations.
 template <int M, int FORCE, bool COMPACT>
-__device__ __forceinline__ double integrate64(const KConst<double>& K,
+__device__ __forceinline__ double integrate64(const KAffine<double>& K,
                                               const aff::LawCoef<double>& c, const double* tab,
                                               const float* __restrict__ U, int n) {
     aff::State<double, M, aff::ALL> s;
@@ -109,7 +109,7 @@ __device__ __forceinline__ double integrate64(const KConst<double>& K,
 // 25 600 steps: 2.08 ms; 2.88 with the conversions in it and one step a
 // loop round.
 template <int M, int FORCE>
-__device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const Coef<float>& cf,
+__device__ __forceinline__ void guess_starts(const KAffine<float>& Kf, const Coef<float>& cf,
                                              const float* rows, int B, double* Y) {
     constexpr int S2 = 2 * M, W = aff::Rows<M, FORCE>::words;
     const aff::LawCoef<float> c = aff::law_coef(cf);
@@ -141,7 +141,7 @@ __device__ __forceinline__ void guess_starts(const KConst<float>& Kf, const Coef
 
 // The start Y[2m] left by guess_starts as (deflections, rates) in FP64.
 template <int M>
-__device__ __forceinline__ void finish_start(const KConst<double>& Kd, double* Y) {
+__device__ __forceinline__ void finish_start(const KAffine<double>& Kd, double* Y) {
     aff::State<float, M, aff::MODE0> s;
     const float2* y = reinterpret_cast<const float2*>(Y);
 #pragma unroll

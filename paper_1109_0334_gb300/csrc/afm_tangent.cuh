@@ -106,7 +106,7 @@ __device__ __forceinline__ float tip(const Tangent<M>& t) {
 // One step of a direction with the primal step's partials P[4] and the
 // direction's own force terms G[4].
 template <int M, int FORCE>
-__device__ __forceinline__ void tangent_step(const KConst<float>& K, const Partials<FORCE>* P,
+__device__ __forceinline__ void tangent_step(const KAffine<float>& K, const Partials<FORCE>* P,
                                              const float* G, Tangent<M>& t) {
     const Affine<float>& A = K.af;
     constexpr bool rate = UsesRate<FORCE>::value;

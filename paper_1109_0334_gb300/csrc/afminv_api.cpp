@@ -16,6 +16,8 @@
 #include "afm_internal.h"
 #include "afm_launch.h"
 
+using afm::AffineFirst;
+using afm::KAffine;
 using afm::KConst;
 
 #include <map>
@@ -351,9 +353,7 @@ void affine_setup(int m, const double* w2, const double* wq, const double* gam, 
 }
 
 template <typename T>
-void fill_kconst(const afm_problem& pr, int spc, int n_steps, KConst<T>& K) {
-    Setup s;
-    modal_setup(pr, spc, s);
+void fill_base(const afm_problem& pr, const Setup& s, int spc, int n_steps, KConst<T>& K) {
     std::memset(&K, 0, sizeof(K));
     const bool drv = pr.drive_mode == 1;
     const double tau = (drv ? pr.dt_s : s.h) / 6.0, nm = 1e-9;
@@ -373,16 +373,6 @@ void fill_kconst(const afm_problem& pr, int spc, int n_steps, KConst<T>& K) {
     K.Zc = (T)(pr.Zc_m / nm);
     K.drive_amp = (s.a / nm) * (s.wd * tau) * (s.wd * tau);
     K.drive_phase = s.psi;
-    if (!drv) {
-        double w2[AFM_MAXM], wq[AFM_MAXM], q0[AFM_MAXM], v0[AFM_MAXM];
-        for (int i = 0; i < s.m; ++i) {
-            w2[i] = (s.w[i] * tau) * (s.w[i] * tau);
-            wq[i] = s.w[i] * tau / pr.Q[i];
-            q0[i] = s.q0[i] / nm;
-            v0[i] = s.v0[i] * tau / nm;
-        }
-        affine_setup(s.m, w2, wq, s.gam, q0, v0, K.drive_amp, K.drive_phase, spc, K.af);
-    }
     K.m = s.m;
     K.spc2 = 2 * spc;
     K.n_steps = n_steps;
@@ -411,6 +401,54 @@ void fill_kconst(const afm_problem& pr, int spc, int n_steps, KConst<T>& K) {
     for (int k = 0; k < pr.n_points && k < AFM_MAX_POINTS; ++k)
         for (int i = 0; i < s.m; ++i)
             K.phi[k][i] = (T)shape_tip_normalised(beam_root(i + 1), pr.point_xi[k]);
+}
+
+// The step's affine map of a problem driven at its own phase table (not of
+// base-motion problems); K's constants are filled.
+template <typename T>
+void fill_map(const afm_problem& pr, const Setup& s, int spc, KAffine<T>& K) {
+    double w2[AFM_MAXM], wq[AFM_MAXM], q0[AFM_MAXM], v0[AFM_MAXM];
+    const double tau = s.h / 6.0, nm = 1e-9;
+    for (int i = 0; i < s.m; ++i) {
+        w2[i] = (s.w[i] * tau) * (s.w[i] * tau);
+        wq[i] = s.w[i] * tau / pr.Q[i];
+        q0[i] = s.q0[i] / nm;
+        v0[i] = s.v0[i] * tau / nm;
+    }
+    affine_setup(s.m, w2, wq, s.gam, q0, v0, K.drive_amp, K.drive_phase, spc, K.af);
+    std::memset(K.AffineFirst<T>::skew, 0, sizeof(K.AffineFirst<T>::skew));
+}
+
+template <typename T>
+void fill_kconst(const afm_problem& pr, KConst<T>& K) {
+    Setup s;
+    modal_setup(pr, pr.steps_per_cycle, s);
+    fill_base(pr, s, pr.steps_per_cycle, pr.n_steps, K);
+}
+
+template <typename T>
+void fill_kaffine(const afm_problem& pr, KAffine<T>& K) {
+    Setup s;
+    modal_setup(pr, pr.steps_per_cycle, s);
+    fill_base(pr, s, pr.steps_per_cycle, pr.n_steps, K);
+    fill_map(pr, s, pr.steps_per_cycle, K);
+}
+
+// Both types' constants of one problem with the maps that are read.
+void fill_pair(const afm_problem& pr, bool map32, bool map64, KAffine<float>& Kf,
+               KAffine<double>& Kd) {
+    Setup s;
+    modal_setup(pr, pr.steps_per_cycle, s);
+    fill_base(pr, s, pr.steps_per_cycle, pr.n_steps, Kf);
+    fill_base(pr, s, pr.steps_per_cycle, pr.n_steps, Kd);
+    if (map32)
+        fill_map(pr, s, pr.steps_per_cycle, Kf);
+    else
+        std::memset(static_cast<AffineFirst<float>*>(&Kf), 0, sizeof(AffineFirst<float>));
+    if (map64)
+        fill_map(pr, s, pr.steps_per_cycle, Kd);
+    else
+        std::memset(static_cast<AffineFirst<double>*>(&Kd), 0, sizeof(AffineFirst<double>));
 }
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
@@ -980,8 +1018,8 @@ PixLayout pix_layout(int n_prob, const afm_problem& pr) {
     L.ld64 = 2 * spc;
     L.ld_rows = spc * afm::aff_row(M, afm::rate_law(pr.force));
     L.kf = 0;
-    L.kd = align256(sizeof(KConst<float>) * n);
-    L.t64 = L.kd + align256(sizeof(KConst<double>) * n);
+    L.kd = align256(sizeof(KAffine<float>) * n);
+    L.t64 = L.kd + align256(sizeof(KAffine<double>) * n);
     L.t32 = L.t64 + align256(sizeof(double) * n * L.ld64);
     L.rows = L.t32 + align256(sizeof(float) * n * L.ld);
     L.total = L.rows + align256(sizeof(float) * n * L.ld_rows);
@@ -1140,18 +1178,17 @@ void trace_push(const char* name) { nvtxRangePushA(name); }
 void trace_pop() { nvtxRangePop(); }
 
 afm_status prepare_invert(afm_ctx* ctx, const afm_problem* prob, const afm_pso_cfg* cfg,
-                          KConst<float>* Kf, KConst<double>* Kd, PsoConst* pc,
+                          KAffine<float>* Kf, KAffine<double>* Kd, PsoConst* pc,
                           size_t* scratch_bytes, size_t* reeval_bytes, int* device) {
     afm_status st = check_problem(prob);
     if (st) return st;
     if ((st = modal_only(prob, "afm_invert_noalloc"))) return st;
     if ((st = check_ctx(ctx))) return st;
     if ((st = check_pso(cfg, prob->n_free))) return st;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, *Kf);
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, *Kd);
     *pc = pso_const(*cfg, prob->n_free);
     *scratch_bytes = invert_layout(cfg->P, prob->n_free).total;
     *reeval_bytes = reeval_extra(*prob);
+    fill_pair(*prob, *reeval_bytes > 0, *reeval_bytes > 0, *Kf, *Kd);
     *device = ctx->device;
     return AFM_OK;
 }
@@ -1286,7 +1323,7 @@ afm_status afm_forward_batch(afm_ctx* ctx, const afm_problem* prob, const float*
         return AFM_OK;
     }
     KConst<float> K;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K);
+    fill_kconst(*prob, K);
     if (prob->drive_mode == 1) {
         AFM_CUDA(timed_launch(ctx, s, [&] { return afm::launch_forward_drive_f32(K, x, P, defl, U, S, s); }),
                  "drive forward kernel");
@@ -1320,16 +1357,17 @@ afm_status afm_forward_batch_f64(afm_ctx* ctx, const afm_problem* prob, const do
         AFM_CUDA(afm::launch_fe_forward_f64(F, x, P, defl, U, S, s), "FE forward f64 kernel");
         return AFM_OK;
     }
-    KConst<double> K;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K);
-    if (prob->drive_mode == 1) {
-        AFM_CUDA(afm::launch_forward_drive_f64(K, x, P, defl, U, S, s), "drive forward f64 kernel");
+    if (prob->drive_mode == 1 || prob->n_points > 0) {
+        KConst<double> K;
+        fill_kconst(*prob, K);
+        if (prob->drive_mode == 1)
+            AFM_CUDA(afm::launch_forward_drive_f64(K, x, P, defl, U, S, s), "drive forward f64 kernel");
+        else
+            AFM_CUDA(afm::launch_forward_points_f64(K, x, P, defl, U, S, s), "points forward f64 kernel");
         return AFM_OK;
     }
-    if (prob->n_points > 0) {
-        AFM_CUDA(afm::launch_forward_points_f64(K, x, P, defl, U, S, s), "points forward f64 kernel");
-        return AFM_OK;
-    }
+    KAffine<double> K;
+    fill_kaffine(*prob, K);
     AFM_CUDA(afm::launch_forward_f64(K, x, P, defl, U, S, nullptr, s), "forward f64 kernel");
     return AFM_OK;
 }
@@ -1508,10 +1546,10 @@ afm_status afm_invert(afm_ctx* ctx, const afm_problem* prob, const float* U,
         AFM_CUDA(afm::launch_fe_invert_final(F, pc, sw, U, history, result, s), "FE invert final kernel");
         return AFM_OK;
     }
-    KConst<float> Kf;
-    KConst<double> Kd;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, Kf);
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, Kd);
+    KAffine<float> Kf;
+    KAffine<double> Kd;
+    const bool reeval = reeval_extra(*prob) > 0;
+    fill_pair(*prob, reeval, reeval, Kf, Kd);
     AFM_CUDA(afm::launch_pso_init(pc, sw, s), "pso init kernel");
     if (prob->drive_mode == 1) {
         for (int it = 0; it <= cfg->iters; ++it)
@@ -1526,7 +1564,7 @@ afm_status afm_invert(afm_ctx* ctx, const afm_problem* prob, const float* U,
                                                : afm::launch_invert_iter(Kf, pc, sw, U, history, it, s);
                  }),
                  "invert iteration kernel");
-    if (reeval_extra(*prob) > 0) {
+    if (reeval) {
         afm::ReevalPtrs R;
         afm::reeval_carve(ws + L.total, problem_modes(*prob), prob->n_steps, prob->steps_per_cycle, &R);
         AFM_CUDA(afm::launch_reeval_pick_swarm(pc, sw, history, R.win, s), "winner pick kernel");
@@ -1569,13 +1607,19 @@ afm_status afm_adjoint(afm_ctx* ctx, const afm_problem* prob, const float* x, in
         sizeof(float) * afm::adjoint_ckpt_floats(problem_modes(*prob), prob->n_steps, P));
     if (workspace_bytes < need)
         return fail(AFM_ERR_INVALID_ARG, "workspace %zu bytes < %zu needed", workspace_bytes, need);
-    KConst<float> K;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    AFM_CUDA(timed_launch(ctx, s, [&] {
-                 return afm::launch_adjoint_split(K, x, P, U, S, dS_dx, static_cast<float*>(workspace),
-                                                  workspace_bytes, s);
-             }),
+    float* ws = static_cast<float*>(workspace);
+    if (afm::adjoint_runs_split(problem_modes(*prob), prob->force, prob->n_steps,
+                                prob->steps_per_cycle, P, workspace, workspace_bytes)) {
+        KAffine<float> K;
+        fill_kaffine(*prob, K);
+        AFM_CUDA(timed_launch(ctx, s, [&] { return afm::launch_adjoint_split(K, x, P, U, S, dS_dx, ws, s); }),
+                 "adjoint kernels");
+        return AFM_OK;
+    }
+    KConst<float> K;
+    fill_kconst(*prob, K);
+    AFM_CUDA(timed_launch(ctx, s, [&] { return afm::launch_adjoint(K, x, P, U, S, dS_dx, ws, s); }),
              "adjoint kernel");
     return AFM_OK;
 }
@@ -1590,8 +1634,8 @@ afm_status afm_normal_equations(afm_ctx* ctx, const afm_problem* prob, const flo
     if ((st = check_ctx(ctx))) return st;
     if (!x || !U || !S || !H || !b || P < 1 || prob->n_free < 1)
         return fail(AFM_ERR_INVALID_ARG, "NULL array, P < 1 or no free parameter");
-    KConst<float> K32;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K32);
+    KAffine<float> K32;
+    fill_kaffine(*prob, K32);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AFM_CUDA(timed_launch(ctx, s, [&] { return afm::launch_sens(K32, x, P, U, S, H, b, s); }),
              "sensitivity kernel");
@@ -1645,7 +1689,7 @@ const double kLmLambda0 = 1e-7, kLmRatio = 10.0;
 // One polish step of Kn candidates x [D][Kn] (S [Kn] receives the misfit at
 // the step's start, then that of the point kept).  Ragged form (off !=
 // nullptr): candidate k is compared with the record of pixel order[k / per].
-afm_status polish_step(afm_ctx* ctx, const KConst<float>& K, int method, const float* U,
+afm_status polish_step(afm_ctx* ctx, const KAffine<float>& K, int method, const float* U,
                        const int64_t* off, const int* order, int per, float* x, float* S, int Kn,
                        int J, const PolishLayout& L, char* ws, cudaStream_t s,
                        const afm::PixConst& pix = afm::PixConst{}) {
@@ -1683,7 +1727,7 @@ afm_status polish_step(afm_ctx* ctx, const KConst<float>& K, int method, const f
     return AFM_OK;
 }
 
-afm_status polish_run(afm_ctx* ctx, const afm_problem& pr, const KConst<float>& K, const float* U,
+afm_status polish_run(afm_ctx* ctx, const afm_problem& pr, const KAffine<float>& K, const float* U,
                       float* x, float* S, int Kn, int steps, int J, int method, char* ws,
                       cudaStream_t s) {
     const PolishLayout L = polish_layout(pr, Kn, J, method, true);
@@ -1743,8 +1787,11 @@ afm_status afm_polish(afm_ctx* ctx, const afm_problem* prob, const float* U, flo
     if (workspace_bytes < need || reinterpret_cast<uintptr_t>(workspace) % 256)
         return fail(AFM_ERR_INVALID_ARG, "workspace too small (%zu < %zu) or misaligned",
                     workspace_bytes, need);
-    KConst<float> K32;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, K32);
+    KAffine<float> K32;
+    if (method == AFM_POLISH_LM)
+        fill_kaffine(*prob, K32);
+    else
+        fill_kconst(*prob, K32);   // the steepest descent reads no map
     return polish_run(ctx, *prob, K32, U, x, S, K, steps, n_cand, method,
                       static_cast<char*>(workspace), reinterpret_cast<cudaStream_t>(stream));
 }
@@ -1801,10 +1848,10 @@ afm_status afm_invert_polished(afm_ctx* ctx, const afm_problem* prob, const floa
     pol += align256(sizeof(float) * (size_t)polish_k);
     int* ik = reinterpret_cast<int*>(pol);
     pol += align256(sizeof(int) * (size_t)polish_k);
-    KConst<float> Kf;
-    KConst<double> Kd;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, Kf);
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, Kd);
+    KAffine<float> Kf;
+    KAffine<double> Kd;
+    const bool reeval = reeval_extra(*prob) > 0;
+    fill_pair(*prob, reeval || method == AFM_POLISH_LM, reeval, Kf, Kd);
     const afm::PsoConst pc = pso_const(*cfg, D);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     AFM_CUDA(afm::launch_pso_init(pc, sw, s), "pso init kernel");
@@ -1817,7 +1864,7 @@ afm_status afm_invert_polished(afm_ctx* ctx, const afm_problem* prob, const floa
     AFM_CUDA(afm::launch_topk(sw.pbS, sw.pb[fin], P, D, polish_k, xk, ik, s), "top-k kernel");
     if ((st = polish_run(ctx, *prob, Kf, U, xk, sk, polish_k, polish_steps, n_cand, method, pol, s)))
         return st;
-    if (reeval_extra(*prob) > 0) {
+    if (reeval) {
         afm::ReevalPtrs R;
         afm::reeval_carve(pol + polish_layout(*prob, polish_k, n_cand, method, true).total, problem_modes(*prob),
                           prob->n_steps, prob->steps_per_cycle, &R);
@@ -1850,8 +1897,8 @@ namespace {
 // the argument block (queue order sorted on `s`), and the particles per
 // thread (forced or autotuned) with the persistent grid size.
 struct BatchSetup {
-    KConst<float> Kf;
-    KConst<double> Kd;
+    KAffine<float> Kf;
+    KAffine<double> Kd;
     afm::PsoConst pc;
     afm::BatchArgs a;
     afm::ReevalBatch R;   // FP64 re-evaluation of the winners (after the queue)
@@ -1883,8 +1930,7 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
     const BatchLayout L = batch_layout(n_run);
     char* ws = static_cast<char*>(workspace);
     BatchSetup& B = *out;
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, B.Kf);
-    fill_kconst(*prob, prob->steps_per_cycle, prob->n_steps, B.Kd);
+    fill_pair(*prob, true, true, B.Kf, B.Kd);
     afm::reeval_batch_carve(ws + L.total, problem_modes(*prob), prob->force, prob->n_steps,
                             prob->steps_per_cycle, n_run, &B.R);
     B.pc = pso_const(*cfg, prob->n_free);
@@ -1917,20 +1963,20 @@ afm_status batch_setup(afm_ctx* ctx, const afm_problem* probs, int n_prob, const
         // and its drive tables computed there
         const PixLayout X = pix_layout(n_prob, *prob);
         char* pw = ws + pix_at;
-        std::vector<KConst<float>> kf(n_prob);
-        std::vector<KConst<double>> kd(n_prob);
+        std::vector<KAffine<float>> kf(n_prob);
+        std::vector<KAffine<double>> kd(n_prob);
         for (int i = 0; i < n_prob; ++i) {
-            fill_kconst(probs[i], prob->steps_per_cycle, prob->n_steps, kf[i]);
-            fill_kconst(probs[i], prob->steps_per_cycle, prob->n_steps, kd[i]);
+            fill_pair(probs[i], true, true, kf[i], kd[i]);
+            kf[i].n_steps = kd[i].n_steps = prob->n_steps;
         }
-        AFM_CUDA(cudaMemcpyAsync(pw + X.kf, kf.data(), sizeof(KConst<float>) * (size_t)n_prob,
+        AFM_CUDA(cudaMemcpyAsync(pw + X.kf, kf.data(), sizeof(KAffine<float>) * (size_t)n_prob,
                                  cudaMemcpyHostToDevice, s),
                  "per-pixel constants upload");
-        AFM_CUDA(cudaMemcpyAsync(pw + X.kd, kd.data(), sizeof(KConst<double>) * (size_t)n_prob,
+        AFM_CUDA(cudaMemcpyAsync(pw + X.kd, kd.data(), sizeof(KAffine<double>) * (size_t)n_prob,
                                  cudaMemcpyHostToDevice, s),
                  "per-pixel constants upload");
-        a.pix.kf = reinterpret_cast<const KConst<float>*>(pw + X.kf);
-        a.pix.kd = reinterpret_cast<const KConst<double>*>(pw + X.kd);
+        a.pix.kf = reinterpret_cast<const KAffine<float>*>(pw + X.kf);
+        a.pix.kd = reinterpret_cast<const KAffine<double>*>(pw + X.kd);
         a.pix.tab64 = reinterpret_cast<const double*>(pw + X.t64);
         a.pix.tab32 = reinterpret_cast<const float*>(pw + X.t32);
         a.pix.rows = reinterpret_cast<const float*>(pw + X.rows);
@@ -1990,8 +2036,8 @@ afm_status afm_invert_batch(afm_ctx* ctx, const afm_problem* probs, int n_prob,
     afm_status st = batch_setup(ctx, probs, n_prob, U_cat, off, n_pix, pixel0, cfg, workspace,
                                 pix_at, results, particles_per_thread, s, "afm_invert_batch", &B);
     if (st) return st;
-    const KConst<float>& Kf = B.Kf;
-    const KConst<double>& Kd = B.Kd;
+    const KAffine<float>& Kf = B.Kf;
+    const KAffine<double>& Kd = B.Kd;
     const afm::PsoConst& pc = B.pc;
     const afm::BatchArgs& a = B.a;
     const int kp = B.kp, grid = B.grid;
@@ -2324,7 +2370,9 @@ afm_status afm_synth_records(afm_ctx* ctx, const afm_problem* prob, const double
                     AFM_TAB_MAX / 2);
     if (!(sigma_m >= 0) || !std::isfinite(sigma_m)) return fail(AFM_ERR_INVALID_ARG, "sigma must be >= 0");
     KConst<float> K;
-    fill_kconst(*prob, prob->steps_per_cycle * sub, prob->n_steps * sub, K);
+    Setup fine;
+    modal_setup(*prob, prob->steps_per_cycle * sub, fine);
+    fill_base(*prob, fine, prob->steps_per_cycle * sub, prob->n_steps * sub, K);
     AFM_CUDA(afm::launch_synth(K, x_truth, n_pix, off, sub, (float)(sigma_m / 1e-9), seed, pixel0,
                                U_cat, reinterpret_cast<cudaStream_t>(stream)),
              "synth kernel");

@@ -463,7 +463,7 @@ __device__ __forceinline__ void reverse_step(const Affine<float>& A, const float
 // terms loaded during the step before (afm_warp.cuh).
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128, 1)
-adj_forward_kernel(const KConst<float> K, const float* __restrict__ x, int P, int ppb,
+adj_forward_kernel(const KAffine<float> K, const float* __restrict__ x, int P, int ppb,
                    const float* __restrict__ U, float* __restrict__ S_out,
                    float* __restrict__ ckpt) {
     constexpr int W = aff::Rows<M, FORCE>::words;
@@ -525,7 +525,7 @@ adj_forward_kernel(const KConst<float> K, const float* __restrict__ x, int P, in
 // segment's sums of the coefficients' cotangents.
 template <int M, int FORCE, bool COEF>
 __global__ void __launch_bounds__(128)
-adj_segment_kernel(const KConst<float> K, const float* __restrict__ x, int P, int nseg,
+adj_segment_kernel(const KAffine<float> K, const float* __restrict__ x, int P, int nseg,
                    const float* __restrict__ U, const float* __restrict__ ckpt, const Recs R) {
     constexpr int NC = aff::CoefDirs<FORCE>::n;
     constexpr int W = aff::Rows<M, FORCE>::words;
@@ -638,7 +638,7 @@ adj_segment_kernel(const KConst<float> K, const float* __restrict__ x, int P, in
 // (c = 2 M) the adjoint state that the segment's residuals give from zero.
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128)
-adj_transfer_kernel(const KConst<float> K, int P, int nseg, const Recs R) {
+adj_transfer_kernel(const KAffine<float> K, int P, int nseg, const Recs R) {
     constexpr int D2 = 2 * M, W = D2 + 1;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long long)nseg * P * W) return;
@@ -770,14 +770,16 @@ size_t adjoint_ws_floats(int m, int force, int n_steps, int P) {
     return std::max(adjoint_ckpt_floats(m, n_steps, P), split);
 }
 
-cudaError_t launch_adjoint_split(const KConst<float>& K, const float* x, int P,
-                                        const float* U, float* S, float* G, float* ckpt,
-                                        size_t ws_bytes, cudaStream_t st) {
-    const int Mt = tmodes(K.m);
-    if (!adj_split(Mt, K.force, K.n_steps, K.spc2 / 2, P) || reinterpret_cast<uintptr_t>(ckpt) % 16 != 0 ||
-        ws_bytes / sizeof(float) < adjoint_ckpt_floats(K.m, K.n_steps, P) +
-                                       split_floats(Mt, rate_law(K.force), K.n_steps, P))
-        return launch_adjoint(K, x, P, U, S, G, ckpt, st);
+bool adjoint_runs_split(int m, int force, int n_steps, int spc, int P, const void* ws,
+                        size_t ws_bytes) {
+    const int M = tmodes(m);
+    return adj_split(M, force, n_steps, spc, P) && reinterpret_cast<uintptr_t>(ws) % 16 == 0 &&
+           ws_bytes / sizeof(float) >= adjoint_ckpt_floats(m, n_steps, P) +
+                                           split_floats(M, rate_law(force), n_steps, P);
+}
+
+cudaError_t launch_adjoint_split(const KAffine<float>& K, const float* x, int P, const float* U,
+                                 float* S, float* G, float* ckpt, cudaStream_t st) {
     const int nseg = (K.n_steps + SEG - 1) / SEG;
     const int ppb = warp::per_block(P), blocks = (P + ppb - 1) / ppb;
     auto per128 = [](long long n) { return (int)((n + 127) / 128); };

@@ -39,8 +39,8 @@ __global__ void pix_tables_kernel(const PixConst pc, int n_pix, int spc2, int wo
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int pix = (int)(t / spc), j = (int)(t % spc);
     if (pix >= n_pix) return;
-    const KConst<float>& kf = pc.kf[pix];
-    const KConst<double>& kd = pc.kd[pix];
+    const KAffine<float>& kf = pc.kf[pix];
+    const KAffine<double>& kd = pc.kd[pix];
     float* t32 = tab32 + (size_t)pix * pc.ld;
     for (int h = 2 * j; h < 2 * j + 2; ++h) {
         const double ph = 6.283185307179586476925 * (double)h / (double)spc2 + kd.drive_phase;

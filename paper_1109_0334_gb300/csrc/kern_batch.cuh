@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(KP == 1 ? 1024 : 512) batch_kernel(const KCons
         if (slot >= a.n_pix) return;
         const int pix = a.order != nullptr ? a.order[slot] : slot;
         if constexpr (PP) {   // this pixel's constants and drive table
-            const unsigned* src = reinterpret_cast<const unsigned*>(a.pix.kf + pix);
+            const KConst<float>* kc = a.pix.kf + pix;   // without the affine map
+            const unsigned* src = reinterpret_cast<const unsigned*>(kc);
             unsigned* dst = reinterpret_cast<unsigned*>(sK);
             for (int w = tid; w < (int)(sizeof(KConst<float>) / 4); w += blockDim.x) dst[w] = src[w];
             const float* t32 = a.pix.tab32 + (size_t)pix * a.pix.ld;

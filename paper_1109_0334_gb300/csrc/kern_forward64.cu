@@ -53,7 +53,7 @@ __device__ __forceinline__ void store_misfit64(double s, double* S, int p, int* 
 
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128)
-fwd64_kernel(const KConst<double> K, const double* __restrict__ x, int P,
+fwd64_kernel(const KAffine<double> K, const double* __restrict__ x, int P,
              double* __restrict__ defl, const double* __restrict__ U, double* __restrict__ S,
              int* __restrict__ flags) {
     extern __shared__ __align__(16) double tab[];
@@ -109,7 +109,7 @@ __device__ __forceinline__ double group_sum64_split(double a, double b, bool odd
 
 template <int M, int FORCE>
 __global__ void __launch_bounds__(128, 1)
-fwd64_lanes_kernel(const KConst<double> K, const double* __restrict__ x, int P, int wpb,
+fwd64_lanes_kernel(const KAffine<double> K, const double* __restrict__ x, int P, int wpb,
                    double* __restrict__ defl, const double* __restrict__ U,
                    double* __restrict__ S, int* __restrict__ flags) {
     constexpr int L = Lanes64<M>::value, G = 32 / L;
@@ -237,7 +237,7 @@ fwd64_lanes_kernel(const KConst<double> K, const double* __restrict__ x, int P, 
     if (S != nullptr && owner) store_misfit64(Sm, S, p, flags);
 }
 
-cudaError_t launch_forward_f64(const KConst<double>& K, const double* x, int P, double* defl,
+cudaError_t launch_forward_f64(const KAffine<double>& K, const double* x, int P, double* defl,
                                const double* U, double* S, int* flags, cudaStream_t st) {
     return dispatch_mf(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
         constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;

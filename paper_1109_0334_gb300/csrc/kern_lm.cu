@@ -54,7 +54,7 @@ constexpr int kFold = 32;   // steps summed in FP32 before folding into FP64 tot
 // ~640 with parameter directions and linearised stages).  16 384 candidates x
 // 1 280 steps: 432 us, 696 us so.
 template <int M, int FORCE, int ND, bool CS, bool PP>
-__global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
+__global__ void __launch_bounds__(kThreads) sens_kernel(const KAffine<float> K0,
                                                         const float* __restrict__ x, int P,
                                                         const float* __restrict__ U,
                                                         const int64_t* __restrict__ off,
@@ -81,13 +81,13 @@ __global__ void __launch_bounds__(kThreads) sens_kernel(const KConst<float> K0,
         U += off[pix];
         n = (int)(off[pix + 1] - off[pix]);
     }
-    const KConst<float>* Kp = &K0;
+    const KAffine<float>* Kp = &K0;
     const float* tab = tabs;
     if constexpr (PP) {
         Kp = pixc.kf + pix;
         tab = pixc.tab32 + (size_t)pix * pixc.ld;
     }
-    const KConst<float>& K = *Kp;
+    const KAffine<float>& K = *Kp;
     const int D = K.D;
     float xd[AFM_MAXD];
     for (int d = 0; d < AFM_MAXD; ++d) xd[d] = d < D ? x[(size_t)d * P + p] : 0.f;
@@ -300,7 +300,7 @@ cudaError_t launch_lm_select_hb(int D, int K, int J, float* x, float* S, double*
     return cudaGetLastError();
 }
 
-cudaError_t launch_sens(const KConst<float>& K, const float* x, int P, const float* U, float* S,
+cudaError_t launch_sens(const KAffine<float>& K, const float* x, int P, const float* U, float* S,
                         double* H, double* b, cudaStream_t st, const int64_t* off, const int* order,
                         int per_slot, const PixConst& pix) {
     const bool pp = pix.kf != nullptr;

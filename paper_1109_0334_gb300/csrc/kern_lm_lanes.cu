@@ -37,7 +37,7 @@ constexpr int kLaneFold = 32;   // as sens_kernel: FP32 blocks of 32 steps folde
 // different lengths; else one record for all.
 template <int M, int FORCE, int ND, bool CS, bool RAG>
 __global__ void __launch_bounds__(kLaneThreads) sens_lanes_kernel(
-    const KConst<float> K, const float* __restrict__ x, int P, const float* __restrict__ U,
+    const KAffine<float> K, const float* __restrict__ x, int P, const float* __restrict__ U,
     const int64_t* __restrict__ off, const int* __restrict__ order, int per_slot, int wpb,
     float* __restrict__ S_out, double* __restrict__ H_out, double* __restrict__ b_out) {
     constexpr int L = ND <= 2 ? 2 : 4, NC = aff::CoefDirs<FORCE>::n;
@@ -197,7 +197,7 @@ bool sens_lanes_preferred(int P, int D) {
     return (long long)P * L <= 152LL * 4 * 32;
 }
 
-cudaError_t launch_sens_lanes(const KConst<float>& K, const float* x, int P, const float* U,
+cudaError_t launch_sens_lanes(const KAffine<float>& K, const float* x, int P, const float* U,
                               float* S, double* H, double* b, cudaStream_t st, const int64_t* off,
                               const int* order, int per_slot) {
     auto byM = [&](auto Mc, auto Fc) -> cudaError_t {

@@ -14,12 +14,12 @@ namespace afm {
 namespace detail {
 afm_status set_error(afm_status st, const char* msg);
 afm_status prepare_invert(afm_ctx* ctx, const afm_problem* prob, const afm_pso_cfg* cfg,
-                          KConst<float>* Kf, KConst<double>* Kd, PsoConst* pc,
+                          KAffine<float>* Kf, KAffine<double>* Kd, PsoConst* pc,
                           size_t* scratch_bytes, size_t* reeval_bytes, int* device);
 void carve_swarm(void* base, int P, int D, SwarmPtrs* sw);
 void clear_error();
-// one fused iteration launch with the context's lanes-per-particle choice,
-// bracketed by the profiling events when afm_profile_enable is on
+// one fused iteration launch, bracketed by the profiling events when
+// afm_profile_enable is on
 cudaError_t invert_iter_timed(afm_ctx* ctx, const KConst<float>& K, const PsoConst& pc,
                               const SwarmPtrs& sw, const float* U, float* history, int it,
                               cudaStream_t s);
@@ -75,8 +75,8 @@ extern "C" afm_status afm_invert_noalloc(afm_ctx* ctx, const afm_problem* prob, 
                                          float* history, void* stream) {
     Trace trace;
     afm::detail::clear_error();
-    afm::KConst<float> Kf;
-    afm::KConst<double> Kd;
+    afm::KAffine<float> Kf;
+    afm::KAffine<double> Kd;
     afm::PsoConst pc;
     size_t need = 0, reeval = 0;
     int device = 0;

@@ -63,8 +63,8 @@ __global__ void reeval_pick_min_kernel(int D, int Kn, const float* __restrict__ 
 // FP32 guess of the segment start states (start[0]; b = 0 is the exact FP64
 // initial state).
 template <int M, int FORCE>
-__global__ void __launch_bounds__(256) reeval_guess_kernel(const KConst<float> Kf,
-                                                           const KConst<double> Kd,
+__global__ void __launch_bounds__(256) reeval_guess_kernel(const KAffine<float> Kf,
+                                                           const KAffine<double> Kd,
                                                            const ReevalPtrs R,
                                                            const float* __restrict__ U) {
     extern __shared__ __align__(16) float tabf[];
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) reeval_guess_kernel(const KConst<float> K
 // segment's misfit share Sb_b; TANGENT: also J_b ([2m][2m], row = output
 // component, column = input direction) in FP32 from the recorded slopes.
 template <int M, int FORCE, bool TANGENT>
-__global__ void __launch_bounds__(32) reeval_pass_kernel(const KConst<double> K,
+__global__ void __launch_bounds__(32) reeval_pass_kernel(const KAffine<double> K,
                                                          const ReevalPtrs R,
                                                          const double* __restrict__ Z,
                                                          const float* __restrict__ U) {
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(32) reeval_correct_kernel(const ReevalPtrs R,
 // S_f64 = sum of the segment shares, the join check (with the sequential
 // fallback) and the result record.  One block of 256.
 template <int M, int FORCE>
-__global__ void __launch_bounds__(256) reeval_final_kernel(const KConst<double> K,
+__global__ void __launch_bounds__(256) reeval_final_kernel(const KAffine<double> K,
                                                            const ReevalPtrs R,
                                                            const double* __restrict__ Z,
                                                            const float* __restrict__ U, int iters,
@@ -307,7 +307,7 @@ cudaError_t launch_reeval_pick_min(int D, int Kn, const float* x, const float* S
     return cudaGetLastError();
 }
 
-cudaError_t launch_reeval(const KConst<float>& Kf, const KConst<double>& Kd, const ReevalPtrs& R,
+cudaError_t launch_reeval(const KAffine<float>& Kf, const KAffine<double>& Kd, const ReevalPtrs& R,
                           const float* U, int iters, const int* flags, void* result,
                           cudaStream_t st) {
     if (!reeval_supported(Kd.m, Kd.n_steps) || R.B != reeval_segments(Kd.n_steps))

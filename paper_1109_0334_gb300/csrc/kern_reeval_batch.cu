@@ -45,7 +45,7 @@ __device__ __forceinline__ int slot_segments(const ReevalBatch& R, int n) {
 // The constants and FP64 drive table of pixel pix: the launch's, or its own
 // (PP: a batch whose pixels differ in their problem).
 template <bool PP, typename T>
-__device__ __forceinline__ const KConst<T>& pix_k(const KConst<T>& K, const KConst<T>* per, int pix) {
+__device__ __forceinline__ const KAffine<T>& pix_k(const KAffine<T>& K, const KAffine<T>* per, int pix) {
     if constexpr (PP)
         return per[pix];
     else
@@ -72,8 +72,8 @@ __device__ __forceinline__ Coef<double> slot_coef(const ReevalBatch& R, int i) {
 }  // namespace
 
 template <int M, int FORCE, bool PP>
-__global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
-                                                       const KConst<double> Kd0,
+__global__ void __launch_bounds__(128) rb_guess_kernel(const KAffine<float> Kf0,
+                                                       const KAffine<double> Kd0,
                                                        const ReevalBatch R, const BatchArgs a) {
     extern __shared__ __align__(16) float tabs[];
     if constexpr (!PP) {
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
     const int i = blockIdx.x * 32 + threadIdx.x;   // warp 0's lanes
     if (threadIdx.x < 32 && i < a.n_pix) {
         const int pix = slot_pixel(a, i);
-        const KConst<float>& Kf = pix_k<PP>(Kf0, a.pix.kf, pix);
-        const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
+        const KAffine<float>& Kf = pix_k<PP>(Kf0, a.pix.kf, pix);
+        const KAffine<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
         const float* tabf = PP ? a.pix.rows + (size_t)pix * a.pix.ld_rows : tabs;
         double xd[AFM_MAXD];
         for (int d = 0; d < AFM_MAXD; ++d) xd[d] = a.res[pix].x[d];
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(128) rb_guess_kernel(const KConst<float> Kf0,
         const int k = blockIdx.x * 32 + w;
         if (k >= a.n_pix) break;
         const int pix = slot_pixel(a, k), B = slot_segments(R, slot_steps(a, pix));
-        const KConst<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
+        const KAffine<double>& Kd = pix_k<PP>(Kd0, a.pix.kd, pix);
         for (int b = 1 + (threadIdx.x & 31); b < B; b += 32)
             finish_start<M>(Kd, R.Z + ((size_t)k * R.maxB + b) * S2);
     }
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128) rb_sumsq_kernel(const ReevalBatch R, cons
 }
 
 template <int M, int FORCE, bool TANGENT, bool PP>
-__global__ void __launch_bounds__(32) rb_pass_kernel(const KConst<double> K0, const ReevalBatch R,
+__global__ void __launch_bounds__(32) rb_pass_kernel(const KAffine<double> K0, const ReevalBatch R,
                                                      const BatchArgs a) {
     __shared__ float rec[TANGENT ? AFM_SEG * kRec * 32 : 1];
     constexpr int S2 = 2 * M;
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(32) rb_pass_kernel(const KConst<double> K0, co
     const int pix = slot_pixel(a, i);
     const int n = slot_steps(a, pix);
     if (b >= slot_segments(R, n)) return;
-    const KConst<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
+    const KAffine<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
     const double* tab = pix_tab64<PP>(R, a, pix);
     const float* U = a.U + a.off[pix];
     const Coef<double> cw = slot_coef(R, i);
@@ -218,14 +218,14 @@ __global__ void __launch_bounds__(128) rb_correct_kernel(const ReevalBatch R, co
 // fallback), and the result record.  One warp per slot (one thread took 750 us
 // for 480 segments, a load after another).
 template <int M, int FORCE, bool PP>
-__global__ void __launch_bounds__(128) rb_final_kernel(const KConst<double> K0, const ReevalBatch R,
+__global__ void __launch_bounds__(128) rb_final_kernel(const KAffine<double> K0, const ReevalBatch R,
                                                        const BatchArgs a) {
     constexpr int S2 = 2 * M;
     const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (i >= a.n_pix) return;
     const int pix = slot_pixel(a, i);
-    const KConst<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
+    const KAffine<double>& K = pix_k<PP>(K0, a.pix.kd, pix);
     const int n = slot_steps(a, pix);
     const int B = slot_segments(R, n);
     const size_t g0 = (size_t)i * R.maxB;
@@ -304,7 +304,7 @@ void reeval_batch_carve(void* base, int m, int force, int n_steps, int spc, int 
     R->maxB = (int)B;
 }
 
-cudaError_t launch_reeval_batch(const KConst<float>& Kf, const KConst<double>& Kd,
+cudaError_t launch_reeval_batch(const KAffine<float>& Kf, const KAffine<double>& Kd,
                                 const ReevalBatch& R, const BatchArgs& a, cudaStream_t st) {
     if (R.maxB != reeval_segments(Kd.n_steps) || Kd.np > 0) return cudaErrorInvalidValue;
     const bool pp = a.pix.kf != nullptr;
