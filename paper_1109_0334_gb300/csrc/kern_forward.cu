@@ -35,23 +35,25 @@ static cudaError_t dispatch_mf(int m, int force, F&& f) {
 // ---------------------------------------------------------------------------
 // Forward + misfit, one thread per particle.
 // ---------------------------------------------------------------------------
-template <typename T, int M, int FORCE>
-__global__ void fwd_kernel(const KConst<T> K, const T* __restrict__ x, int P,
-                           T* __restrict__ defl, const T* __restrict__ U, T* __restrict__ S,
-                           int* __restrict__ flags) {
+constexpr int FWD_THREADS = 128;
+
+template <int M, int FORCE>
+__global__ void __launch_bounds__(FWD_THREADS) fwd_kernel(const KConst<float> K, const float* __restrict__ x, int P,
+                           float* __restrict__ defl, const float* __restrict__ U,
+                           float* __restrict__ S, int* __restrict__ flags) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* tab = reinterpret_cast<T*>(smem_raw);
+    float* tab = reinterpret_cast<float*>(smem_raw);
     build_drive_table(K, tab);
     __syncthreads();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= P) return;
-    T xd[AFM_MAXD];
+    float xd[AFM_MAXD];
     for (int d = 0; d < K.D; ++d) xd[d] = x[(size_t)d * P + p];
-    Coef<T> c = make_coef<T, T>(K, xd);
-    T s = integrate<T, M, FORCE>(K, c, tab, U, defl, P, p, K.n_steps);
+    const Coef<float> c = make_coef<float, float>(K, xd);
+    float s = integrate<float, M, FORCE>(K, c, tab, U, defl, P, p, K.n_steps);
     if (S != nullptr) {
-        if (!(s < (T)INFINITY)) {
-            s = (T)INFINITY;
+        if (!(s < INFINITY)) {
+            s = INFINITY;
             if (flags != nullptr) atomicAdd(flags, 1);
         }
         S[p] = s;
@@ -150,21 +152,14 @@ static cudaError_t launch_forward_x2(const KConst<float>& K, const float* x, int
     return go(std::integral_constant<int, 3>{});
 }
 
-template <typename T>
-static cudaError_t launch_forward(const KConst<T>& K, const T* x, int P, T* defl, const T* U,
-                                  T* S, int* flags, cudaStream_t st) {
-    const int threads = P <= 152 * 32 * 4 ? 32 : 128;
-    const int blocks = (P + threads - 1) / threads;
-    const size_t smem = sizeof(T) * (size_t)(K.spc2 + 1);
+// More particles than one warp per SM sub-partition.
+static cudaError_t launch_forward(const KConst<float>& K, const float* x, int P, float* defl,
+                                  const float* U, float* S, int* flags, cudaStream_t st) {
+    const int blocks = (P + FWD_THREADS - 1) / FWD_THREADS;
+    const size_t smem = sizeof(float) * (size_t)(K.spc2 + 1);
     return dispatch_mf(K.m, K.force, [&](auto Mc, auto Fc) -> cudaError_t {
-        constexpr int M = decltype(Mc)::value, FORCE = decltype(Fc)::value;
-        auto kern = fwd_kernel<T, M, FORCE>;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        kern<<<blocks, threads, smem, st>>>(K, x, P, defl, U, S, flags);
+        fwd_kernel<decltype(Mc)::value, decltype(Fc)::value>
+            <<<blocks, FWD_THREADS, smem, st>>>(K, x, P, defl, U, S, flags);
         return cudaGetLastError();
     });
 }
@@ -182,7 +177,7 @@ cudaError_t launch_forward_f32(const KConst<float>& K, const float* x, int P, fl
             return cudaGetLastError();
         });
     }
-    return launch_forward<float>(K, x, P, defl, U, S, flags, st);
+    return launch_forward(K, x, P, defl, U, S, flags, st);
 }
 
 // ---------------------------------------------------------------------------
