@@ -349,26 +349,39 @@ size_t split_floats(int M, bool rate, int n_steps, int P) {
 // step, and costs five more launches (~55 us) and the work of the maps' 2 M + 1
 // columns and the way back, ~0.05 ns x P a step and column, which the one
 // kernel's idle SMs would not have done.  Measured, one kernel / split:
-//   few particles (32): 160 steps 0.96 .. 1.27, 200 1.08 .. 1.45, 256 1.2 ..
-//     1.6, 512 1.7 .. 2.4, 2500 3.1 .. 4.0
-//   break-even particles at 256 / 512 / 1000 steps: 1 mode (DMT) 1750 / 3800 /
-//     5800, 3 modes (DMT + KV, spring-damper) 2400 / 3300 / 4000, 8 modes
-//     (spring-damper) 1800 / 2100 / past 2222
+//   few particles (32): 128 steps 0.8 (1 mode) .. 1.15 (8), 160 0.96 .. 1.27,
+//     200 1.08 .. 1.45, 256 1.2 .. 1.6, 512 1.7 .. 2.4, 2500 3.1 .. 4.0
+//   break-even particles at 200 / 256 / 512 / 1000 steps: 1 mode (DMT) 700 /
+//     1600 / 3800 / 5800; 3 modes (DMT and DMT + KV) 2000 / 2300 / 3700 / 5000,
+//     (spring-damper) 4000 at 1000; 8 modes (Hooke) past 2222 from 256 on,
+//     (spring-damper) 1450 / 1800 / 2100 / 2300
 //   its blocks build their drive rows, which shows past 512 phases: at 1280
 //     steps 3 modes break even at 4000 particles with 1024 phases and 2700 with
 //     2048, 8 modes (spring-damper) past 1700 and at 1400
-// The lines below stay within those: 0.99 at their worst, where the start of
-// the range meets one mode.
-long long split_max_particles(int M, int n_steps) {
-    const long long most = M == 1 ? 6000 : (M == 3 ? 4000 : 1700);
-    return std::max(0ll, std::min({most, 12 * (n_steps - 180ll), 2000 + 2ll * n_steps}));
+// The lines below stay within those (0.97 at their worst).
+long long split_max_particles(int M, int force, int n_steps) {
+    const long long n = n_steps;
+    const bool rate = rate_law(force), kv = force == F_DMT_KV;
+    long long most, rise, flat = 2000 + 12 * n / 5;
+    if (M == 1) {   // DMT + KV: the one kernel's step is 1.3 times DMT's
+        most = rate && !kv ? 4500 : 6000;
+        rise = kv ? 20 * (n - 150) : 12 * (n - (rate ? 155 : 170));
+        if (kv) flat = 2500 + 3 * n;
+    } else if (M == 3) {
+        most = rate ? 4000 : 5000;
+        rise = rate ? 18 * (n - 140) : 17 * (n - 130);
+    } else {
+        most = rate ? 1500 + n / 2 : 2222;
+        rise = rate ? 13 * (n - 130) : 15 * (n - 110);
+    }
+    return std::max(0ll, std::min({most, rise, flat}));
 }
 
 // Its records stay within 256 MB.
 constexpr size_t SPLIT_FLOATS = 64u << 20;
 
 bool adj_split(int M, int force, int n_steps, int spc, int P) {
-    return P <= split_max_particles(M, n_steps) && (long long)P * spc <= (M <= 3 ? 4000000 : 1500000) &&
+    return P <= split_max_particles(M, force, n_steps) && (long long)P * spc <= (M <= 3 ? 4000000 : 1500000) &&
            split_floats(M, rate_law(force), n_steps, P) <= SPLIT_FLOATS;
 }
 
@@ -764,7 +777,7 @@ size_t adjoint_ckpt_floats(int m, int n_steps, int P) {
 // longer record's size serves a smaller one's split form too.
 size_t adjoint_ws_floats(int m, int force, int n_steps, int P) {
     const int M = tmodes(m);
-    const int Ps = (int)std::min((long long)P, split_max_particles(M, n_steps));
+    const int Ps = (int)std::min((long long)P, split_max_particles(M, force, n_steps));
     const size_t split = adjoint_ckpt_floats(m, n_steps, Ps) +
                          std::min(split_floats(M, rate_law(force), n_steps, Ps), SPLIT_FLOATS);
     return std::max(adjoint_ckpt_floats(m, n_steps, P), split);

@@ -40,9 +40,9 @@ def test_size_is_monotone(afm, load, modes):
 
 @pytest.mark.parametrize("load,modes", [("c1", 1), ("c2", 3), ("f2_hooke", 8)])
 def test_short_records_take_the_checkpoints_alone(afm, load, modes):
-    """The segments at once are slower than the one kernel below ~180 steps
-    (0.2 to 0.9 of its speed at 128), whatever the batch."""
-    for n in (1, 32, 128, 180):
+    """The segments at once are slower than the one kernel below ~110 steps
+    (0.2 to 0.9 of its speed at 64), whatever the batch."""
+    for n in (1, 32, 64, 110):
         prob = afm.make_problem(W.get(load, n_modes=modes), n_steps=n)
         for P in (1, 700, 10000):
             assert afm.adjoint_workspace_size(prob, P) == _checkpoints(n, modes, P), (n, P)

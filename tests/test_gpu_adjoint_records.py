@@ -1,5 +1,5 @@
 """Both forms of the adjoint on records long enough for the segments at once
-(kern_adjoint.cu: more than 180 steps), chosen by the workspace: S and G of
+(kern_adjoint.cu: more than 110 to 170 steps), chosen by the workspace: S and G of
 each against the oracle's complex step.  Step counts around the 32-step
 segments, particle counts up to the form's bound for them."""
 import numpy as np
