@@ -385,16 +385,19 @@ afm_status afm_invert_polished(afm_ctx* ctx, const afm_problem* prob, const floa
  * on `stream` before the launch (the call returns once they are staged),
  * and pixel i's result equals afm_invert on probs[i] alone bit for bit.
  * One persistent kernel: blocks pull pixels from a queue, longest record
- * first, and keep the whole swarm of a pixel on chip; then every winner is
+ * first (or, where every pixel has a resident block, are dealt one by the SM
+ * they run on), and keep the whole swarm of a pixel on chip; then every winner is
  * re-evaluated in FP64.  results [n_pix] (device afm_result) are indexed by
  * pixel.  The launch sequence is captured once into a CUDA graph (cached in
  * the context per argument set) and replayed on `stream`.
  * Particles per thread: *particles_per_thread = 1, 2 or 4 forces a choice;
  * NULL or 0 selects the autotuner, which on the first call for a new (modes,
- * force, P, D, steps per cycle) times one evaluation of the first wave of
+ * force, P, D, steps per cycle) and number of pixels per SM (to a factor of
+ * two, and past the resident blocks) times one evaluation of the first wave of
  * pixels per candidate (synchronous: make that call before any capture of
- * `stream`), scales it by the waves the batch needs at that candidate's
- * occupancy and caches the fastest in the context.  With 2 or 4 particles
+ * `stream`; a captured call takes the choice of the nearest number of pixels),
+ * scales it by the waves the batch needs at that candidate's occupancy and
+ * caches the fastest in the context.  With 2 or 4 particles
  * per thread, DMT swarms step two particles per paired FP32 instruction
  * (bit-identical to one per thread).  The choice used is written back to
  * *particles_per_thread if non-NULL.

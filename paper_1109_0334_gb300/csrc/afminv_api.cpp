@@ -37,13 +37,18 @@ struct afm_batch_graph {
     cudaEvent_t ev_own[2];
 };
 
+struct afm_batch_choice {
+    int max_occ;              // resident blocks per SM, of the candidate with most
+    std::map<int, int> kp;    // by load
+};
+
 struct afm_ctx {
     int device;
     int num_sms;
     // afm_invert_batch: particles per thread chosen by the autotuner, per
     // (modes, force, particles, free parameters, steps per cycle, per-pixel
-    // problems)
-    std::map<std::tuple<int, int, int, int, int, int>, int> batch_kp;
+    // problems) and load (batch_load)
+    std::map<std::tuple<int, int, int, int, int, int>, afm_batch_choice> batch_kp;
     cudaStream_t capture_stream = nullptr;
     std::vector<afm_batch_graph> batch_graphs;
     // kernel timing (afm_profile_*): events around each fused iteration launch
@@ -1070,17 +1075,54 @@ void append_bytes(std::vector<unsigned char>& v, const T& x) {
     v.insert(v.end(), p, p + sizeof(T));
 }
 
+// How many pixels share an SM: 0 for one at most, then a step per doubling, and
+// one more past the resident blocks, where blocks pull pixels from a queue.  A
+// few pixels are bound by one block's chain (one particle per thread), many by
+// the SMs' throughput, so a choice timed at one load is not another's.
+int batch_load(int n_pix, int num_sms, int max_occ) {
+    int b = 0;
+    while (((long long)num_sms << b) < n_pix && (1 << b) < max_occ) ++b;
+    return n_pix > (long long)num_sms * max_occ ? b + 1 : b;
+}
+
 // Autotuner of afm_invert_batch: times one swarm evaluation of the first wave
 // of pixels for each particles-per-thread choice and keeps the one with the
 // lowest estimated batch time (the wave's time x the waves the batch needs).
+// A captured stream cannot be timed: it takes the choice of the nearest load.
 afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst& pc,
                       const afm::BatchArgs& a, bool selected, cudaStream_t s, int* kp_out,
                       int* occ_out) {
     const bool pp = a.pix.kf != nullptr;
     const auto key = std::make_tuple(Kf.m, Kf.force, pc.P, pc.D, Kf.spc2, (int)pp);
+    auto occupancy = [&](int kp) {   // 0: not a candidate
+        int occ = 0;
+        if (afm::batch_threads(pc.P, kp) > afm::batch_max_threads(kp) || (kp > 1 && Kf.m > 3)) return 0;
+        if (afm::batch_occupancy(Kf.m, Kf.force, kp, pc.P, pc.D, Kf.spc2, pp, &occ) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        return occ;
+    };
     auto it = ctx->batch_kp.find(key);
-    if (it != ctx->batch_kp.end()) {
-        *kp_out = it->second;
+    if (it == ctx->batch_kp.end()) {
+        afm_batch_choice c{0, {}};
+        for (int kp : {1, 2, 4}) c.max_occ = std::max(c.max_occ, occupancy(kp));
+        if (c.max_occ < 1)
+            return fail(AFM_ERR_UNSUPPORTED, "no batch kernel configuration fits P = %d", pc.P);
+        it = ctx->batch_kp.emplace(key, c).first;
+    }
+    std::map<int, int>& known = it->second.kp;
+    const int load = batch_load(a.n_pix, ctx->num_sms, it->second.max_occ);
+    auto hit = known.find(load);
+    if (hit == known.end() && !known.empty()) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) cudaGetLastError();
+        if (cs != cudaStreamCaptureStatusNone)
+            for (auto k = known.begin(); k != known.end(); ++k)
+                if (hit == known.end() || std::abs(k->first - load) < std::abs(hit->first - load)) hit = k;
+    }
+    if (hit != known.end()) {
+        *kp_out = hit->second;
         AFM_CUDA(afm::batch_occupancy(Kf.m, Kf.force, *kp_out, pc.P, pc.D, Kf.spc2, pp, occ_out),
                  "batch occupancy");
         return AFM_OK;
@@ -1102,18 +1144,16 @@ afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst
     AFM_CUDA(cudaEventCreate(&e0), "cudaEventCreate");
     AFM_CUDA(cudaEventCreate(&e1), "cudaEventCreate");
     for (int kp : {1, 2, 4}) {
-        const int threads = afm::batch_threads(pc.P, kp);
-        if (threads > afm::batch_max_threads(kp) || (kp > 1 && Kf.m > 3)) continue;
-        int occ = 0;
-        if (afm::batch_occupancy(Kf.m, Kf.force, kp, pc.P, pc.D, Kf.spc2, pp, &occ) != cudaSuccess ||
-            occ < 1) {
-            cudaGetLastError();
-            continue;
-        }
+        const int occ = occupancy(kp);
+        if (occ < 1) continue;
         afm::PsoConst probe = pc;
         probe.iters = 0;
         afm::BatchArgs pa = a;
         pa.n_pix = std::min(a.n_pix, ctx->num_sms * occ);
+        // dealt, also where the batch will pull from the queue: a queue of many
+        // more pixels evens the SMs out as dealing does one wave (timed as one
+        // wave of the queue, 4096 pixels of 20 to 200 cycles got 1 particle per
+        // thread, 970 ms, for 2, 938)
         pa.layer = ctx->num_sms;
         const int grid = pa.n_pix;
         AFM_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int) * afm::batch_queue_words(a.n_pix), s), "cudaMemsetAsync");
@@ -1146,8 +1186,7 @@ afm_status batch_tune(afm_ctx* ctx, const KConst<float>& Kf, const afm::PsoConst
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best_kp == 0) return fail(AFM_ERR_UNSUPPORTED, "no batch kernel configuration fits P = %d", pc.P);
-    ctx->batch_kp[key] = best_kp;
+    known[load] = best_kp;
     *kp_out = best_kp;
     *occ_out = best_occ;
     return AFM_OK;
