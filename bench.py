@@ -87,21 +87,27 @@ def fe_algo_ops_per_step(n: int = 64) -> int:
     return 8 * n + 27
 
 
-def fe_fp32_ops_per_step() -> int:
+def fe_fp32_ops_per_step(particles: int) -> int:
     """FP32 add/mul/fma instructions per particle per step of the FP32 FE
-    kernel (DMT law, 64 modes on 8 lanes of 8 mode slots), counted from its
-    source.  Per lane: the force history term 1; slot 0 (compensated): the
-    increment 5 (drive and past-force terms 2, state terms 2, b1's low word
-    1), the predicted coordinate 3, the update 1 + 8 (two Kahan sums); slots
-    1-7: delta + increment 4, the predicted coordinate 1, the update 2; the
-    lane's tip tree 7 and the group's sum 3; one Newton step 15 (gap 1 + law
-    4.5, residual 2, update 2, gap 1 + law 4.5; the law's constant products
-    hoisted, contact and free branches 5 and 4).  Lane 0 alone: the tip
-    deflection and the compensated misfit 6."""
-    slot0 = 5 + 3 + 1 + 8
+    kernel (DMT law, 64 modes), counted from its source.  A launch gives a
+    particle 4 lanes of 16 mode slots or 8 of 8, by its warps per SM
+    sub-partition (kern_fe.cu); the lowest 8 modes are compensated.  Per lane:
+    the force history term 1; a compensated slot: the increment 5 (drive and
+    past-force terms 2, state terms 2, b1's low word 1), the predicted
+    coordinate 3, the update 1 + 8 (two Kahan sums); a plain slot: delta +
+    increment 4, the predicted coordinate 1, the update 2; the lane's tip sum
+    (slots - 1) and the group's (log2 of the lanes); one Newton step 15 (gap 1
+    + law 4.5, residual 2, update 2, gap 1 + law 4.5; the law's constant
+    products hoisted, contact and free branches 5 and 4).  Lane 0 alone: the
+    tip deflection and the compensated misfit 6.  666 on 4 lanes, 742 on 8."""
+    warps = (particles + 2431) // 2432
+    lanes = 4 if warps == 2 or warps >= 4 else 8
+    slots, comp = 64 // lanes, 8 // lanes
+    slot_comp = 5 + 3 + 1 + 8
     slot_plain = 4 + 1 + 2
-    per_lane = 1 + slot0 + 7 * slot_plain + 7 + 3 + 15
-    return 8 * per_lane + 6
+    per_lane = (1 + comp * slot_comp + (slots - comp) * slot_plain + (slots - 1)
+                + lanes.bit_length() - 1 + 15)
+    return lanes * per_lane + 6
 
 
 # ---------------------------------------------------------------------------
@@ -646,7 +652,7 @@ def run_c5(A, W, dev, peak_ops, flush, iters=None):
             "roofline": {"bound": "alu", "achieved": ach / 1e12, "peak": peak_ops / 1e12,
                          "unit": "T FP32 lane-ops/s", "frac": ach / peak_ops,
                          "ops_per_particle_step": ops_ps,
-                         "issued_ops_per_particle_step": fe_fp32_ops_per_step(),
+                         "issued_ops_per_particle_step": fe_fp32_ops_per_step(spec["P"]),
                          "kernel": "fe_modal_kernel<float,DMT,invert iteration>",
                          "traffic": ncu_traffic("fe_modal_kernel", "c5"),
                          "note": "modal-basis Newmark kernel (no dense propagator)"}}
@@ -759,21 +765,6 @@ def run_points(A, W, dev, flush):
         out[label] = {"ms_per_inversion": e0.elapsed_time(e1), "record_values": int(U.numel()),
                       "ident_rel_err_vs_truth": ident_errors(list(r["theta"]), th_t)[:3],
                       "S_f64_nm2": r["S_f64"], "status": r["status"]}
-    # the same three-point inversion on the one-lane kernel (bit-identical)
-    prob, cfg, U = A.make_problem(spec), A.make_pso(spec), rec.reshape(-1)
-    A.set_lanes("one")
-    try:
-        flush.zero_()
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        res, _ = A.invert(prob, U, cfg)
-        e1.record()
-        e1.synchronize()
-    finally:
-        A.set_lanes("auto")
-    r = A.decode_result(res)
-    out["three_points_one_lane"] = {"ms_per_inversion": e0.elapsed_time(e1),
-                                    "same_result": r["S_f64"] == out["three_points"]["S_f64_nm2"]}
     out["ident"] = "H R, E* sqrt(R), a0"
     return out
 
