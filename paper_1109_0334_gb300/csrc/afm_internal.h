@@ -108,7 +108,8 @@ struct KConst {
     // The arrays start 8 bytes past a 16-byte boundary, here and in KAffine: on
     // one, the compiler reads them 16 bytes at a time into more registers, and
     // the eight-mode kernels were slower (DMT, 19 457 particles x 512 steps 220
-    // us, 211 so; Hooke's sensitivities, 512 x 512 steps, 212 us, 196 so).
+    // us, 211 so; Hooke's sensitivities, 512 x 512 steps, 212 us, 196 so).  The
+    // batch kernel's copy in shared memory has them on one.
     double skew;
     T w2[AFM_MAXM], w2lo[AFM_MAXM], wq[AFM_MAXM], gam[AFM_MAXM], tip[AFM_MAXM];
     T q0[AFM_MAXM], v0[AFM_MAXM];
@@ -155,7 +156,7 @@ static_assert(sizeof(KAffine<float>) == sizeof(KConst<float>) + sizeof(Affine<fl
 // f_i = (h^2/4) k phi_i(tip) / s_i (force in units of k * 1 nm); the tip
 // deflection is sum_i phi_i(tip) z_i.
 #define AFM_FE_MAXN 64      // DOFs = modes (2 per node)
-#define AFM_FE_LANES 8      // lanes per particle in the FE kernels
+#define AFM_FE_LANES 8      // lowest modes with compensated sums in FP32 (the 8-lane layout's slot 0)
 
 struct FeConst {
     int ne, n, spc, n_steps;

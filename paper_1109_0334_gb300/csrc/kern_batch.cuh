@@ -2,6 +2,8 @@
 // kern_batch.cu); instantiated per force law in kern_batch_*.cu so that the
 // translation units compile in parallel.
 #pragma once
+#include <stddef.h>
+
 #include "../../include/afminv.h"
 #include "afm_device.cuh"
 #include "afm_f32x2.cuh"
@@ -85,10 +87,15 @@ __device__ __forceinline__ int any_left(const BatchArgs& a) {
 }  // namespace batch_detail
 
 // 32-bit words of dynamic shared memory before the drive table (per-pixel
-// constants), a multiple of 4 so that the arrays after it stay 16-byte aligned
+// constants), a multiple of 4 so that the arrays after it stay 16-byte aligned.
+// The constants start KC_AT words in, which puts their arrays on 16-byte
+// boundaries: a step reads them in fewer loads (4096 pixels, 7 evaluations, 4
+// particles per thread: 869 ms, 922 eight bytes off).
+constexpr int KC_AT = 2;
+static_assert((4 * KC_AT + offsetof(KConst<float>, w2)) % 16 == 0, "arrays of the constants");
 template <bool PP>
 __host__ __device__ constexpr int batch_kc_words() {
-    return PP ? (int)((sizeof(KConst<float>) + 15) / 16 * 4) : 0;
+    return PP ? (int)((4 * KC_AT + sizeof(KConst<float>) + 15) / 16 * 4) : 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -101,7 +108,7 @@ __global__ void __launch_bounds__(KP == 1 ? 1024 : 512) batch_kernel(const KCons
                                                      const BatchArgs a) {
     extern __shared__ __align__(16) float sm[];
     const int P = pc.P, D = pc.D;
-    KConst<float>* sK = reinterpret_cast<KConst<float>*>(sm);
+    KConst<float>* sK = reinterpret_cast<KConst<float>*>(sm + KC_AT);
     float* tab = sm + batch_kc_words<PP>();
     float* sx = tab + ((K.spc2 + 1 + 3) & ~3);
     float* sv = sx + D * P;
