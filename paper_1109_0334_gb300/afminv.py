@@ -182,9 +182,10 @@ LANES = {"auto": 0, "one": 1, "stages": 2, "modes2": 3, "modes4": 4, "modes3": 5
 
 
 def set_lanes(lanes: str = "auto", device=None) -> None:
-    """Lanes per particle of the fused inversion iteration (see afm_set_lanes):
-    'auto', 'one', 'stages', 'modes2', 'modes3' or 'modes4'; all are
-    bit-identical."""
+    """Particle layout (see afm_set_lanes): 'one' keeps one particle per thread
+    in forward_batch's large DMT batches, which otherwise run two.  The
+    inversions run one lane per particle whatever the value ('auto', 'one',
+    'stages', 'modes2', 'modes3' or 'modes4'); all are bit-identical."""
     _check(lib().afm_set_lanes(context(device), LANES[lanes]))
 
 

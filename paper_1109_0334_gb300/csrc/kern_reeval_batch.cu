@@ -4,8 +4,9 @@
 // own record in segments of AFM_SEG steps.  Slot i owns segments
 // [i * maxB, i * maxB + B_i), B_i = ceil(n_i / AFM_SEG), maxB that of the
 // longest record; threads past B_i return at once.
-//   guess    one thread per slot: FP32 run of the winner (the swarm kernels'
-//            compensated step), keeping the state at every segment start;
+//   guess    one thread per slot: FP32 run of the winner (the affine step with
+//            mode 0 compensated; the swarms run the stage form), keeping the
+//            state at every segment start;
 //   sweep    (twice) one thread per segment: FP64 integration from its start
 //            with the FP32 tangent map; one warp per slot walks its joins;
 //   final    the FP64 pass from the corrected starts sums each segment's
